@@ -64,7 +64,7 @@ typedef enum felbm_status {
 #define FELBM_MESH_GENERAL 0x4u /* never use the structured-lattice kernels */
 #define FELBM_PERIODIC_Z 0x8u   /* tetrahedral meshes: box[2] > 0 is the period in z */
 #define FELBM_MESH_SPLIT_STEP 0x10u /* general triangle meshes: always four launches per step */
-#define FELBM_MESH_PATCH_STEP 0x20u /* general triangle meshes: always the one-launch patch step */
+#define FELBM_MESH_PATCH_STEP 0x20u /* general triangle meshes: the two-launch patch step (the default) */
 
 /* precision of the stored distributions and of the bulk arithmetic */
 #define FELBM_FP64 0
@@ -118,12 +118,11 @@ typedef struct felbm_params {
  * The library computes element geometry, the lumped mass, the assembled
  * streaming/recovery coefficients and an internal node order: patches of
  * 256 nodes along a Hilbert curve over the domain, reverse Cuthill-McKee
- * order within a patch.  A general mesh of up to 2^18 nodes steps in one
- * launch per step, one block per patch with the patch's nodes up to 4 edges
- * away staged in shared memory; larger ones in four launches per step over
- * global fields (measured faster there).  FELBM_MESH_SPLIT_STEP and
- * FELBM_MESH_PATCH_STEP force one of the two; both give the same results bit
- * for bit.  A mesh that is the structured split of a unit lattice
+ * order within a patch.  A general mesh steps in two launches per step: the
+ * streamed h and rho, then one block per patch with the patch's nodes up to
+ * 3 edges away staged in shared memory.  FELBM_MESH_SPLIT_STEP asks for four
+ * launches per step over global fields instead (as does a mesh whose patches
+ * do not fit shared memory); both give the same results bit for bit.  A mesh that is the structured split of a unit lattice
  * (node i at ((i mod nx) h, (i div nx) h), each square cut along its
  * (i,j)-(i+1,j+1) diagonal, periodic in x, periodic or walled in y) is served
  * by the structured-lattice kernels unless FELBM_MESH_GENERAL is set.
@@ -275,7 +274,7 @@ void felbm_batch_destroy(felbm_batch *batch);
  *   0 stream h + rho, 1 grad rho, 2 lap rho / stress / mu,
  *   3 grad mu + stream + collide (the general four-pass step),
  *   4 lattice step (one launch per step on structured meshes),
- *   5 patch step (one launch per step on general triangle meshes),
+ *   5 patch step (second launch per step on general triangle meshes, after 0),
  *   6-7 unused. */
 #define FELBM_PROFILE_KINDS 8
 

@@ -53,24 +53,63 @@ int cuda_status(cudaError_t e) {
     } while (0)
 
 template <typename T>
-static DevCSR<T> dev_csr(const felbm_mesh *m) {
-    DevCSR<T> d;
+static DevELL<T> dev_ell(const felbm_mesh *m) {
+    DevELL<T> d;
     d.n = (int32_t)m->n_nodes;
-    d.rowptr = m->d_rowptr;
-    d.col = m->d_col;
-    const size_t nnz = m->host.col.size();
-    const T *base;
-    if (sizeof(T) == 8)
-        base = reinterpret_cast<const T *>(m->d_coef64);
-    else
-        base = reinterpret_cast<const T *>(m->d_coef32);
-    d.ax = base;
-    d.ay = base + nnz;
-    d.bxx = base + 2 * nnz;
-    d.bxy = base + 3 * nnz;
-    d.byy = base + 4 * nnz;
+    d.sbase = m->d_sbase;
+    void *const *e = m->d_ell[sizeof(T) == 8];
+    d.a = reinterpret_cast<const Ell2<T> *>(e[0]);
+    d.b = reinterpret_cast<const Ell2<T> *>(e[1]);
+    d.c = reinterpret_cast<const Ell2<T> *>(e[2]);
+    d.deg = m->d_deg;
     d.tag = m->d_tag;
     return d;
+}
+
+std::vector<int32_t> ell_slices(int32_t n, const std::vector<int32_t> &rowptr) {
+    std::vector<int32_t> sb((size_t)(n + 31) / 32 + 1, 0);
+    for (size_t s = 0; s + 1 < sb.size(); ++s) {
+        int32_t w = 0;
+        for (int32_t i = (int32_t)(32 * s); i < std::min<int64_t>(n, 32 * (int64_t)(s + 1)); ++i)
+            w = std::max(w, rowptr[i + 1] - rowptr[i]);
+        sb[s + 1] = sb[s] + w;
+    }
+    return sb;
+}
+
+cudaError_t mesh_upload(felbm_mesh *m, void **d, const void *host, size_t bytes) {
+    cudaError_t e = cudaMalloc(d, std::max<size_t>(bytes, 1));
+    if (e != cudaSuccess) return e;
+    m->device_bytes += (int64_t)bytes;
+    return bytes ? cudaMemcpy(*d, host, bytes, cudaMemcpyHostToDevice) : cudaSuccess;
+}
+
+// The entries of DevELL<T> (slices sb) from the assembled rows.
+template <typename T>
+static cudaError_t upload_ell(felbm_mesh *m, const std::vector<int32_t> &sb) {
+    const HostCSR &H = m->host;
+    const size_t entries = (size_t)sb.back() * 32;
+    std::vector<Ell2<T>> a(entries), b(entries), c(entries);
+    for (size_t s = 0; s + 1 < sb.size(); ++s)
+        for (int32_t k = 0; k < sb[s + 1] - sb[s]; ++k)
+            for (int32_t l = 0; l < 32; ++l) {
+                const size_t p = ((size_t)sb[s] + k) * 32 + l;
+                const int64_t i = std::min<int64_t>(32 * (int64_t)s + l, H.n - 1);
+                const int64_t q = (int64_t)H.rowptr[i] + k;
+                if (q < H.rowptr[i + 1]) {
+                    a[p] = {(T)H.ax[q], (T)H.ay[q]};
+                    b[p] = {(T)H.bxx[q], (T)H.bxy[q]};
+                    c[p] = {(T)H.byy[q], ell_id<T>(H.col[q])};
+                } else {
+                    a[p] = b[p] = {T(0), T(0)};
+                    c[p] = {T(0), ell_id<T>((int32_t)i)};
+                }
+            }
+    void **d = m->d_ell[sizeof(T) == 8];
+    cudaError_t e = mesh_upload(m, &d[0], a.data(), entries * sizeof(Ell2<T>));
+    if (e == cudaSuccess) e = mesh_upload(m, &d[1], b.data(), entries * sizeof(Ell2<T>));
+    if (e == cudaSuccess) e = mesh_upload(m, &d[2], c.data(), entries * sizeof(Ell2<T>));
+    return e;
 }
 
 template <typename T>
@@ -151,10 +190,13 @@ static DevLattice<T> dev_lattice(const felbm_mesh *m) {
 // Derivative chain shared by init and step: rho (already in F.rho) ->
 // grad rho -> lap rho, K, mu.
 // Threads per block of the general path's node kernels (one node per
-// thread).  On the 256 x 256 Delaunay mesh (65,536 nodes, fewer blocks than
-// two per SM) blocks of 128 and 64 threads spread the mesh more evenly but
-// ran 3-7% slower than 256.
-constexpr int kGenBlock = 256;
+// thread).
+constexpr int kGenBlock = 128;
+
+// Whether a general mesh's patches are all resident at once at two blocks
+// per SM (152 SMs): its step is then bound by latency, and its kernels take
+// more registers per thread.
+constexpr int64_t kOneWave = 2 * 152 * kPatch;
 
 // kappa in FP64 (the FP64 kappa lap rho term of FELBM_PARAM_LAP_FP64)
 static double kappa64(const felbm_params &p) {
@@ -165,7 +207,7 @@ static double kappa64(const felbm_params &p) {
 static bool lap_fp64(const felbm_state *s) { return s->esize == 4 && (s->params.flags & FELBM_PARAM_LAP_FP64); }
 
 // The mesh's operators with FP64 coefficients, for the FP64 Laplacian.
-static DevCSR<double> topo64(const felbm_mesh *m, const DevCSR<float> &) { return dev_csr<double>(m); }
+static DevELL<double> topo64(const felbm_mesh *m, const DevELL<float> &) { return dev_ell<double>(m); }
 static DevLattice<double> topo64(const felbm_mesh *m, const DevLattice<float> &) { return dev_lattice<double>(m); }
 
 template <typename T, typename Topo>
@@ -175,44 +217,48 @@ static void launch_chain(felbm_state *s, const Topo &d) {
     const Phys<T> P = phys_of<T>(s->params);
     const unsigned g = nblocks(m->n_nodes, kGenBlock);
     int sl = prof_begin(s, 1);
-    k_grad<T, Topo><<<g, kGenBlock, 0, m->stream>>>(d, F);
+    launch_pdl(k_grad<T, Topo>, g, kGenBlock, 0, m->stream, d, F);
     prof_end(s, sl);
     sl = prof_begin(s, 2);
     if constexpr (sizeof(T) == 4) {
         if (lap_fp64(s)) {
             const auto d64 = topo64(m, d);
-            k_mu_lap64<decltype(d64)><<<g, kGenBlock, 0, m->stream>>>(d64, F, P, kappa64(s->params));
+            launch_pdl(k_mu_lap64<std::decay_t<decltype(d64)>>, g, kGenBlock, 0, m->stream, d64, F, P, kappa64(s->params));
         } else {
-            k_mu<T, Topo><<<g, kGenBlock, 0, m->stream>>>(d, F, P);
+            launch_pdl(k_mu<T, Topo>, g, kGenBlock, 0, m->stream, d, F, P);
         }
     } else {
-        k_mu<T, Topo><<<g, kGenBlock, 0, m->stream>>>(d, F, P);
+        launch_pdl(k_mu<T, Topo>, g, kGenBlock, 0, m->stream, d, F, P);
     }
     prof_end(s, sl);
+}
+
+// The first launch of a general mesh's step: streamed h* and rho.
+template <typename T, typename Topo>
+static CollideArgs<T, Topo> step_rho(felbm_state *s, const Topo &d, bool write_mom) {
+    const felbm_mesh *m = s->mesh;
+    CollideArgs<T, Topo> A;
+    A.m = d;
+    A.fin = reinterpret_cast<const T *>(s->f[s->cur]);
+    A.fout = reinterpret_cast<T *>(s->f[s->cur ^ 1]);
+    A.F = fields_of<T>(s);
+    A.P = phys_of<T>(s->params);
+    A.mom = write_mom ? reinterpret_cast<T *>(s->mom) : nullptr;
+    A.flag = s->d_flag;
+    const int sl = prof_begin(s, 0);
+    launch_pdl(m->n_nodes <= kOneWave ? k_rho<T, Topo, true> : k_rho<T, Topo, false>,
+               nblocks(m->n_nodes, kGenBlock), kGenBlock, 0, m->stream, d, A.fin, A.P.dt, A.F.rho, A.F.hs);
+    prof_end(s, sl);
+    return A;
 }
 
 template <typename T, typename Topo>
 static void step_topo(felbm_state *s, const Topo &d, bool write_mom) {
     const felbm_mesh *m = s->mesh;
-    const Fields<T> F = fields_of<T>(s);
-    const Phys<T> P = phys_of<T>(s->params);
-    const unsigned g = nblocks(m->n_nodes, kGenBlock);
-    const T *fin = reinterpret_cast<const T *>(s->f[s->cur]);
-    T *fout = reinterpret_cast<T *>(s->f[s->cur ^ 1]);
-    int sl = prof_begin(s, 0);
-    k_rho<T, Topo><<<g, kGenBlock, 0, m->stream>>>(d, fin, P.dt, F.rho, F.hs);
-    prof_end(s, sl);
+    const CollideArgs<T, Topo> A = step_rho<T, Topo>(s, d, write_mom);
     launch_chain<T, Topo>(s, d);
-    CollideArgs<T, Topo> A;
-    A.m = d;
-    A.fin = fin;
-    A.fout = fout;
-    A.F = F;
-    A.P = P;
-    A.mom = write_mom ? reinterpret_cast<T *>(s->mom) : nullptr;
-    A.flag = s->d_flag;
-    sl = prof_begin(s, 3);
-    k_collide<T, Topo><<<g, kGenBlock, 0, m->stream>>>(A);
+    const int sl = prof_begin(s, 3);
+    launch_pdl(k_collide<T, Topo>, nblocks(m->n_nodes, kGenBlock), kGenBlock, 0, m->stream, A);
     prof_end(s, sl);
     s->cur ^= 1;
 }
@@ -294,43 +340,42 @@ static cudaError_t lat_smem_attr() {
     return cudaSuccess;
 }
 
-// One launch per step over the patches of a general triangle mesh; false
-// when its shared memory exceeds what a block can have (the four-launch
-// step then runs).
+// Two launches per step over a general triangle mesh with patches; false
+// when the patch kernel's shared memory exceeds what a block can have (the
+// four-launch step then runs).
 template <typename T, bool LAP64>
 static bool patch_steps(felbm_state *s, int64_t n, cudaError_t &err) {
     const felbm_mesh *m = s->mesh;
     const HostCSR &H = m->host;
-    const size_t smem = patch_smem<T>(H.rmax, H.r1max, H.r2max, H.r3max);
+    using CT = typename std::conditional<LAP64, double, T>::type;
+    const size_t smem = patch_smem<T, CT>(H.r1max, H.r2max, H.r3max, H.pemax, H.psmax);
     if (smem > 227 * 1024) return false;
-    err = cudaFuncSetAttribute(k_patch_step<T, LAP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kernel = m->n_nodes <= kOneWave ? k_patch_step<T, LAP64, true> : k_patch_step<T, LAP64, false>;
+    err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) {
         cudaGetLastError();
         return true;
     }
+    const DevELL<T> d = dev_ell<T>(m);
     PatchArgs<T> A;
-    A.m = dev_csr<T>(m);
     A.nbase = m->d_pnbase;
     A.count = m->d_pcount;
     A.node = m->d_pnode;
-    A.rowbase = m->d_prowbase;
-    A.lcol = m->d_plcol;
-    A.rmax = H.rmax;
+    A.pslice = m->d_pslice;
+    A.psbase = m->d_psbase;
+    A.pcol = m->d_pcol;
+    A.pa = m->d_pa[sizeof(CT) == 8];
     A.r1max = H.r1max;
     A.r2max = H.r2max;
     A.r3max = H.r3max;
-    A.P = phys_of<T>(s->params);
-    A.flag = s->d_flag;
-    A.ax64 = m->d_coef64;  // SoA: a_x, a_y, b_xx, b_xy, b_yy
-    A.ay64 = m->d_coef64 + m->host.col.size();
+    A.pemax = H.pemax;
+    A.psmax = H.psmax;
     A.kappa64 = kappa64(s->params);
     const unsigned blocks = (unsigned)(H.pnbase.size() - 1);
     for (int64_t k = 0; k < n; ++k) {
-        A.fin = reinterpret_cast<const T *>(s->f[s->cur]);
-        A.fout = reinterpret_cast<T *>(s->f[s->cur ^ 1]);
-        A.mom = k == n - 1 ? reinterpret_cast<T *>(s->mom) : nullptr;
+        A.c = step_rho<T>(s, d, k == n - 1);
         const int sl = prof_begin(s, 5);
-        k_patch_step<T, LAP64><<<blocks, kPatch, smem, m->stream>>>(A);
+        launch_pdl(kernel, blocks, kPatch, smem, m->stream, A);
         prof_end(s, sl);
         s->cur ^= 1;
     }
@@ -386,7 +431,7 @@ static int do_steps(felbm_state *s, int64_t n) {
             step_lattice<T, false>(s, A, k == n - 1);
         }
     } else {
-        const DevCSR<T> d = dev_csr<T>(m);
+        const DevELL<T> d = dev_ell<T>(m);
         for (int64_t k = 0; k < n; ++k) step_topo<T>(s, d, k == n - 1);
     }
     return FELBM_OK;
@@ -397,7 +442,7 @@ static void init_any(felbm_state *s) {
     if (s->mesh->kind == 1)
         init_topo<T>(s, dev_lattice<T>(s->mesh));
     else
-        init_topo<T>(s, dev_csr<T>(s->mesh));
+        init_topo<T>(s, dev_ell<T>(s->mesh));
 }
 
 template <typename T>
@@ -415,18 +460,20 @@ static void launch_moments(felbm_state *s) {
 
 void mesh_free(felbm_mesh *m) {
     if (!m) return;
-    cudaFree(m->d_rowptr);
-    cudaFree(m->d_col);
+    cudaFree(m->d_sbase);
+    cudaFree(m->d_deg);
+    for (auto &p : m->d_ell)
+        for (void *q : p) cudaFree(q);
     cudaFree(m->d_perm);
-    cudaFree(m->d_coef64);
-    cudaFree(m->d_coef32);
     cudaFree(m->d_mass);
     cudaFree(m->d_tag);
     cudaFree(m->d_pnbase);
     cudaFree(m->d_pcount);
     cudaFree(m->d_pnode);
-    cudaFree(m->d_prowbase);
-    cudaFree(m->d_plcol);
+    cudaFree(m->d_pslice);
+    cudaFree(m->d_psbase);
+    cudaFree(m->d_pcol);
+    for (void *q : m->d_pa) cudaFree(q);
     delete m;
 }
 
@@ -552,7 +599,7 @@ int felbm_mesh_create(const double *xy, int64_t n_nodes, const int32_t *tri, int
     }
     m->kind = m->sinfo.ok ? 1 : 0;
     const HostCSR &H = m->host;
-    const size_t N = (size_t)n_nodes, nnz = H.col.size();
+    const size_t N = (size_t)n_nodes;
     cudaError_t e = cudaSuccess;
     auto alloc = [&](void **p, size_t bytes) {
         if (e == cudaSuccess) {
@@ -562,24 +609,9 @@ int felbm_mesh_create(const double *xy, int64_t n_nodes, const int32_t *tri, int
     };
     alloc((void **)&m->d_mass, N * sizeof(double));
     if (m->kind == 0) {
-        alloc((void **)&m->d_rowptr, (N + 1) * sizeof(int32_t));
-        alloc((void **)&m->d_col, nnz * sizeof(int32_t));
         alloc((void **)&m->d_perm, 2 * N * sizeof(int32_t));
-        alloc((void **)&m->d_coef64, 5 * nnz * sizeof(double));
-        alloc((void **)&m->d_coef32, 5 * nnz * sizeof(float));
         if (!H.tag.empty()) alloc((void **)&m->d_tag, N);
-        // the patch step by default up to kPatchStepMaxNodes (measured: 1.48x
-        // faster on 65,536 nodes, even on 262,144, 1.27x slower on 1,048,576,
-        // where its dependent coefficient loads leave it latency-bound)
-        m->patch_step = !H.pnbase.empty() && ((flags & FELBM_MESH_PATCH_STEP) ||
-                                              (!(flags & FELBM_MESH_SPLIT_STEP) && n_nodes <= kPatchStepMaxNodes));
-        if (m->patch_step) {
-            alloc((void **)&m->d_pnbase, H.pnbase.size() * sizeof(int32_t));
-            alloc((void **)&m->d_pcount, H.pcount.size() * sizeof(int32_t));
-            alloc((void **)&m->d_pnode, H.pnode.size() * sizeof(int32_t));
-            alloc((void **)&m->d_prowbase, H.prowbase.size() * sizeof(int32_t));
-            alloc((void **)&m->d_plcol, std::max<size_t>(H.plcol.size(), 1) * sizeof(uint16_t));
-        }
+        m->patch_step = !H.pnbase.empty() && !(flags & FELBM_MESH_SPLIT_STEP);
     }
     if (e != cudaSuccess) {
         int rs = cuda_status(e);
@@ -593,36 +625,42 @@ int felbm_mesh_create(const double *xy, int64_t n_nodes, const int32_t *tri, int
     } else {
         e = cudaMemcpy(m->d_mass, H.mass.data(), N * sizeof(double), cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
-            e = cudaMemcpy(m->d_rowptr, H.rowptr.data(), (N + 1) * sizeof(int32_t), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(m->d_col, H.col.data(), nnz * sizeof(int32_t), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
             e = cudaMemcpy(m->d_perm, H.perm.data(), N * sizeof(int32_t), cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
             e = cudaMemcpy(m->d_perm + N, H.iperm.data(), N * sizeof(int32_t), cudaMemcpyHostToDevice);
-        std::vector<double> c64(5 * nnz);
-        std::vector<float> c32(5 * nnz);
-        const std::vector<double> *src[5] = {&H.ax, &H.ay, &H.bxx, &H.bxy, &H.byy};
-        for (int k = 0; k < 5; ++k)
-            for (size_t q = 0; q < nnz; ++q) {
-                c64[k * nnz + q] = (*src[k])[q];
-                c32[k * nnz + q] = (float)(*src[k])[q];
-            }
-        if (e == cudaSuccess)
-            e = cudaMemcpy(m->d_coef64, c64.data(), 5 * nnz * sizeof(double), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(m->d_coef32, c32.data(), 5 * nnz * sizeof(float), cudaMemcpyHostToDevice);
         if (e == cudaSuccess && m->d_tag)
             e = cudaMemcpy(m->d_tag, H.tag.data(), N, cudaMemcpyHostToDevice);
-        if (m->patch_step) {
+        try {
             auto up = [&](void *d, const void *h, size_t b) {
-                if (e == cudaSuccess && b) e = cudaMemcpy(d, h, b, cudaMemcpyHostToDevice);
+                if (e == cudaSuccess) e = mesh_upload(m, (void **)d, h, b);
             };
-            up(m->d_pnbase, H.pnbase.data(), H.pnbase.size() * sizeof(int32_t));
-            up(m->d_pcount, H.pcount.data(), H.pcount.size() * sizeof(int32_t));
-            up(m->d_pnode, H.pnode.data(), H.pnode.size() * sizeof(int32_t));
-            up(m->d_prowbase, H.prowbase.data(), H.prowbase.size() * sizeof(int32_t));
-            up(m->d_plcol, H.plcol.data(), H.plcol.size() * sizeof(uint16_t));
+            const std::vector<int32_t> sb = ell_slices(H.n, H.rowptr);
+            std::vector<uint8_t> deg(N);
+            for (size_t k = 0; k < N; ++k) deg[k] = (uint8_t)std::min(255, H.rowptr[k + 1] - H.rowptr[k]);
+            up(&m->d_sbase, sb.data(), sb.size() * sizeof(int32_t));
+            up(&m->d_deg, deg.data(), N);
+            if (e == cudaSuccess) e = upload_ell<float>(m, sb);
+            if (e == cudaSuccess) e = upload_ell<double>(m, sb);
+            if (m->patch_step) {
+                up(&m->d_pnbase, H.pnbase.data(), H.pnbase.size() * sizeof(int32_t));
+                up(&m->d_pcount, H.pcount.data(), H.pcount.size() * sizeof(int32_t));
+                up(&m->d_pnode, H.pnode.data(), H.pnode.size() * sizeof(int32_t));
+                up(&m->d_pslice, H.pslice.data(), H.pslice.size() * sizeof(int32_t));
+                up(&m->d_psbase, H.psbase.data(), H.psbase.size() * sizeof(int32_t));
+                up(&m->d_pcol, H.pcol.data(), H.pcol.size() * sizeof(uint16_t));
+                const size_t ne = H.pcsr.size();
+                std::vector<float> a32(2 * ne, 0.0f);
+                std::vector<double> a64(2 * ne, 0.0);
+                for (size_t k = 0; k < ne; ++k)
+                    if (H.pcsr[k] >= 0) {
+                        a32[2 * k] = (float)(a64[2 * k] = H.ax[H.pcsr[k]]);
+                        a32[2 * k + 1] = (float)(a64[2 * k + 1] = H.ay[H.pcsr[k]]);
+                    }
+                up(&m->d_pa[0], a32.data(), 2 * ne * sizeof(float));
+                up(&m->d_pa[1], a64.data(), 2 * ne * sizeof(double));
+            }
+        } catch (const std::bad_alloc &) {
+            e = cudaErrorMemoryAllocation;
         }
     }
     if (e != cudaSuccess) {

@@ -1,6 +1,7 @@
 // C ABI on tetrahedral meshes (D3Q19; kind 2 general CSR, kind 3 Kuhn
 // lattice): mesh creation and the per-state work the common entry points of
 // felbm_api.cu hand over here.
+#include <algorithm>
 #include <cmath>
 #include <new>
 #include <type_traits>
@@ -26,17 +27,47 @@ static size_t pop_index3(int a, size_t i, size_t n) {
 }
 
 template <typename T>
-static DevCSR3<T> dev_csr3(const felbm_mesh *m) {
-    DevCSR3<T> d;
+static DevELL3<T> dev_ell3(const felbm_mesh *m) {
+    DevELL3<T> d;
     d.n = (int32_t)m->n_nodes;
-    d.rowptr = m->d_rowptr;
-    d.col = m->d_col;
-    const size_t nnz = m->host3.col.size();
-    const T *base = sizeof(T) == 8 ? reinterpret_cast<const T *>(m->d_coef64)
-                                   : reinterpret_cast<const T *>(m->d_coef32);
-    for (int k = 0; k < 9; ++k) d.c[k] = base + (size_t)k * nnz;
+    d.sbase = m->d_sbase;
+    void *const *e = m->d_ell[sizeof(T) == 8];
+    d.a = reinterpret_cast<const Ell4<T> *>(e[0]);
+    d.b = reinterpret_cast<const Ell4<T> *>(e[1]);
+    d.c = reinterpret_cast<const Ell2<T> *>(e[2]);
     d.tag = m->d_tag;
     return d;
+}
+
+// The entries of DevELL3<T> (slices sb) from the assembled rows.
+template <typename T>
+static cudaError_t upload_ell3(felbm_mesh *m, const std::vector<int32_t> &sb) {
+    const HostCSR3 &H = m->host3;
+    const size_t entries = (size_t)sb.back() * 32, nnz = H.col.size();
+    const double *cf = H.coef.data();
+    std::vector<Ell4<T>> a(entries), b(entries);
+    std::vector<T> c(2 * entries, T(0));
+    for (size_t s = 0; s + 1 < sb.size(); ++s)
+        for (int32_t k = 0; k < sb[s + 1] - sb[s]; ++k)
+            for (int32_t l = 0; l < 32; ++l) {
+                const size_t p = ((size_t)sb[s] + k) * 32 + l;
+                const int64_t i = std::min<int64_t>(32 * (int64_t)s + l, H.n - 1);
+                const int64_t q = (int64_t)H.rowptr[i] + k;
+                if (q < H.rowptr[i + 1]) {
+                    a[p] = {(T)cf[q], (T)cf[nnz + q], (T)cf[2 * nnz + q], ell_id<T>(H.col[q])};
+                    b[p] = {(T)cf[3 * nnz + q], (T)cf[4 * nnz + q], (T)cf[5 * nnz + q], (T)cf[6 * nnz + q]};
+                    c[2 * p] = (T)cf[7 * nnz + q];
+                    c[2 * p + 1] = (T)cf[8 * nnz + q];
+                } else {
+                    a[p] = {T(0), T(0), T(0), ell_id<T>((int32_t)i)};
+                    b[p] = {T(0), T(0), T(0), T(0)};
+                }
+            }
+    void **d = m->d_ell[sizeof(T) == 8];
+    cudaError_t e = mesh_upload(m, &d[0], a.data(), entries * sizeof(Ell4<T>));
+    if (e == cudaSuccess) e = mesh_upload(m, &d[1], b.data(), entries * sizeof(Ell4<T>));
+    if (e == cudaSuccess) e = mesh_upload(m, &d[2], c.data(), 2 * entries * sizeof(T));
+    return e;
 }
 
 template <typename T>
@@ -116,7 +147,7 @@ static void with_topo(felbm_state *s, Fn &&fn) {
     if (s->mesh->kind == 3)
         fn(dev_lat3<T>(s->mesh, s->params.dt));
     else
-        fn(dev_csr3<T>(s->mesh));
+        fn(dev_ell3<T>(s->mesh));
 }
 
 template <typename T>
@@ -358,7 +389,7 @@ extern "C" int felbm_mesh_create_tet(const double *xyz, int64_t n_nodes, const i
         std::vector<double>().swap(H.coef);
         std::vector<uint8_t>().swap(H.tag);
     }
-    const size_t N = (size_t)n_nodes, nnz = H.col.size();
+    const size_t N = (size_t)n_nodes;
     cudaError_t e = cudaSuccess;
     auto alloc = [&](void **p, size_t bytes) {
         if (e == cudaSuccess) {
@@ -369,32 +400,22 @@ extern "C" int felbm_mesh_create_tet(const double *xyz, int64_t n_nodes, const i
     const bool csr = m->kind == 2;
     alloc((void **)&m->d_mass, N * sizeof(double));
     alloc((void **)&m->d_perm, 2 * N * sizeof(int32_t));
-    if (csr) {
-        alloc((void **)&m->d_rowptr, (N + 1) * sizeof(int32_t));
-        alloc((void **)&m->d_col, nnz * sizeof(int32_t));
-        alloc((void **)&m->d_coef64, 9 * nnz * sizeof(double));
-        alloc((void **)&m->d_coef32, 9 * nnz * sizeof(float));
-        if (!H.tag.empty()) alloc((void **)&m->d_tag, N);
-    }
-    std::vector<float> c32;
-    try {
-        c32.resize(9 * nnz);
-    } catch (const std::bad_alloc &) {
-        e = cudaErrorMemoryAllocation;
-    }
-    for (size_t q = 0; q < c32.size(); ++q) c32[q] = (float)H.coef[q];
+    if (csr && !H.tag.empty()) alloc((void **)&m->d_tag, N);
     if (e == cudaSuccess) e = cudaMemcpy(m->d_mass, H.mass.data(), N * sizeof(double), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && csr)
-        e = cudaMemcpy(m->d_rowptr, H.rowptr.data(), (N + 1) * sizeof(int32_t), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && csr)
-        e = cudaMemcpy(m->d_col, H.col.data(), nnz * sizeof(int32_t), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->d_perm, H.perm.data(), N * sizeof(int32_t), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(m->d_perm + N, H.iperm.data(), N * sizeof(int32_t), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && csr)
-        e = cudaMemcpy(m->d_coef64, H.coef.data(), 9 * nnz * sizeof(double), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && csr)
-        e = cudaMemcpy(m->d_coef32, c32.data(), 9 * nnz * sizeof(float), cudaMemcpyHostToDevice);
+    if (csr) {
+        try {
+            const std::vector<int32_t> sb = ell_slices(H.n, H.rowptr);
+            if (e == cudaSuccess)
+                e = mesh_upload(m, (void **)&m->d_sbase, sb.data(), sb.size() * sizeof(int32_t));
+            if (e == cudaSuccess) e = upload_ell3<float>(m, sb);
+            if (e == cudaSuccess) e = upload_ell3<double>(m, sb);
+        } catch (const std::bad_alloc &) {
+            e = cudaErrorMemoryAllocation;
+        }
+    }
     if (e == cudaSuccess && m->d_tag) e = cudaMemcpy(m->d_tag, H.tag.data(), N, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         const int rs = cuda_status(e);

@@ -5,6 +5,7 @@
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
 
+#include <utility>
 #include <vector>
 
 #include "../../include/felbm.h"
@@ -50,6 +51,35 @@ struct NvtxRange {
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
+// ---- programmatic dependent launch -----------------------------------------
+// The kernels of a step are launched with programmatic stream serialisation:
+// a kernel may start while its predecessor drains, reads only what no kernel
+// writes (mesh tables) before pdl_wait(), and everything else after it.
+// pdl_wait() returns once the predecessor has completed, which itself waited
+// for its own, so the order of all memory accesses is that of plain launches.
+// Kernels trigger only after their wait, so that at most two of them are
+// resident at a time.  What other kernels write is read with plain loads:
+// the compiler may move non-coherent ones (__ldg, const __restrict__) ahead
+// of the wait.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A &&...args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+#endif
+
 unsigned check_bits_api();
 unsigned check_bits_api3();
 unsigned check_bits_batch();
@@ -72,20 +102,21 @@ struct HostCSR {
     std::vector<uint8_t> tag;      // internal order, empty if no walls
     std::vector<int32_t> perm;     // perm[internal] = caller id
     std::vector<int32_t> iperm;    // iperm[caller] = internal id
-    // Patches of the one-launch step (internal order is patch-major: patch p
-    // owns the nodes [p kPatch, min(n, (p + 1) kPatch))).  Per patch its
-    // region: its own nodes, then the nodes 1, 2, 3 and 4 edges away, as
-    // internal ids in pnode[pnbase[p] ..); pcount[4 p ..] the cumulative
-    // counts of rings <= 0, 1, 2, 3.  For the region nodes of rings <= 3,
-    // prowbase gives the offset in plcol of the region indices of their CSR
-    // columns (in CSR order).
-    std::vector<int32_t> pnbase, pcount, pnode, prowbase;
-    std::vector<uint16_t> plcol;
-    int32_t rmax = 0, r1max = 0, r2max = 0, r3max = 0;  // largest region / ring <= 1, 2, 3 sizes
+    // Patches (internal order is patch-major: patch p owns the nodes
+    // [p kPatch, min(n, (p + 1) kPatch))).  Per patch its region: its own
+    // nodes, then the nodes 1, 2 and 3 edges away, as internal ids in
+    // pnode[pnbase[p] ..); pcount[4 p ..] the counts of rings <= 0, 1, 2, 3.
+    // The rows of rings <= 2 lie in slices of 32 (as DevELL's): pslice[p]
+    // is the patch's first entry of psbase, which holds its slices' first
+    // rows of 32 entries (one more than it has slices); pcol has the region
+    // index and pcsr the CSR entry of each (-1: padding, index of the row).
+    std::vector<int32_t> pnbase, pcount, pnode, pslice, psbase, pcsr;
+    std::vector<uint16_t> pcol;
+    int32_t r1max = 0, r2max = 0, r3max = 0;  // largest ring <= 1, 2, 3 sizes
+    int32_t pemax = 0, psmax = 0;             // most rows of 32 entries, most slices of a patch
 };
 
-constexpr int kPatch = 256;  // nodes per patch of the general one-launch step
-constexpr int64_t kPatchStepMaxNodes = 1 << 18;  // default patch step up to this size
+constexpr int kPatch = 256;  // nodes per patch of general triangle meshes
 
 // General tetrahedral mesh (3-D), same conventions: for each neighbour j != i
 // a_ij = sum_{T∋i,j} |T| grad N_j / (4 m_i) (3 components) and the symmetric
@@ -171,27 +202,136 @@ void detect_structured(const double *xy, int64_t n_nodes, const int32_t *tri, in
 
 // ---- device-side views --------------------------------------------------
 
-// Neighbour topologies.  for_each(i, fn) calls fn(j, ax, ay, bxx, bxy, byy)
+// Neighbour topologies.  each(row(i), fn) calls fn(j, ax, ay, bxx, bxy, byy)
 // for every neighbour j != i of node i with the assembled coefficients a_ij,
 // b_ij; tag_of(i) is the wall tag (0 = fluid).
 
-// General mesh: CSR in reverse Cuthill-McKee order.
+// Rows of a general mesh in slices of 32 nodes (a warp's), internal order:
+// slice s holds rows sbase[s] .. sbase[s+1] of 32 entries, row k the k-th
+// neighbour of each of its nodes, in the order of the CSR row.  A warp's
+// loads of one row are then consecutive 16- and 8-byte words: against CSR
+// arrays, where lanes step by a whole row, a pass over the rows touches a
+// sixth of the cache lines.  Entries past a node's degree hold the node
+// itself and zero coefficients; they are not read.
 template <typename T>
-struct DevCSR {
-    int32_t n;
-    const int32_t *rowptr;
-    const int32_t *col;
-    const T *ax, *ay, *bxx, *bxy, *byy;
-    const uint8_t *tag;  // nullptr if no walls
+struct alignas(2 * sizeof(T)) Ell2 {
+    T x, y;
+};
+template <typename T>
+struct alignas(16) Ell4 {
+    T x, y, z, w;
+};
 #ifdef __CUDACC__
-    template <typename Fn>
-    __device__ __forceinline__ void for_each(int32_t i, Fn &&fn) const {
-        const int32_t p1 = __ldg(rowptr + i + 1);
-        for (int32_t p = __ldg(rowptr + i); p < p1; ++p) {
-            const int32_t j = __ldg(col + p);
-            if (!chk_idx(j, n, 1u)) continue;
-            fn(j, __ldg(ax + p), __ldg(ay + p), __ldg(bxx + p), __ldg(bxy + p), __ldg(byy + p));
+#define FELBM_HD __host__ __device__
+#else
+#define FELBM_HD
+#endif
+// a node id in a T (its bits, or its value in FP64), and back
+template <typename T>
+FELBM_HD inline T ell_id(int32_t c) {
+    if (sizeof(T) == 8) return (T)c;
+    union {
+        int32_t i;
+        float f;
+    } u;
+    u.i = c;
+    return (T)u.f;
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ Ell2<float> ell_load(const Ell2<float> *p) {
+    const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
+    return {v.x, v.y};
+}
+__device__ __forceinline__ Ell2<double> ell_load(const Ell2<double> *p) {
+    const double2 v = __ldg(reinterpret_cast<const double2 *>(p));
+    return {v.x, v.y};
+}
+__device__ __forceinline__ Ell4<float> ell_load(const Ell4<float> *p) {
+    const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
+    return {v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ Ell4<double> ell_load(const Ell4<double> *p) {
+    const double2 a = __ldg(reinterpret_cast<const double2 *>(p)), b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
+    return {a.x, a.y, b.x, b.y};
+}
+__device__ __forceinline__ int32_t ell_get(float w) { return __float_as_int(w); }
+__device__ __forceinline__ int32_t ell_get(double w) { return __double2int_rn(w); }
+#endif
+
+// General triangle mesh: {a_x, a_y}, {b_xx, b_xy} and {b_yy, neighbour}.
+// row(i) reads the first entries of node i, which no kernel writes;
+// each(row, fn) calls fn(j, ax, ay, bxx, bxy, byy) for all of them, in
+// chunks.  Within a chunk the code has no branch, so that all its gathers are
+// in flight at once: a pass waits for one L2 access per chunk and not per
+// neighbour.
+template <typename T>
+struct DevELL {
+    static constexpr int kChunk = sizeof(T) == 4 ? 4 : 2;
+    int32_t n;
+    const int32_t *sbase;
+    const Ell2<T> *a, *b, *c;
+    const uint8_t *deg;   // neighbours of each node (255: as many as its slice has rows)
+    const uint8_t *tag;   // nullptr if no walls
+#ifdef __CUDACC__
+    struct Chunk {
+        Ell2<T> a[kChunk], b[kChunk], c[kChunk];
+    };
+    struct Row {
+        size_t p;  // first entry
+        int32_t i, deg;
+        Chunk k[2];
+    };
+    // entries k0 .. k0 + kChunk - 1 of a row (A: with a)
+    template <bool A>
+    __device__ __forceinline__ void load(size_t p, int32_t i, int32_t deg, int k0, Chunk &r) const {
+#pragma unroll
+        for (int k = 0; k < kChunk; ++k) {
+            r.a[k] = r.b[k] = {T(0), T(0)};
+            r.c[k] = {T(0), ell_id<T>(i)};
+            if (k0 + k < deg) {
+                const size_t e = p + 32 * (k0 + k);
+                if (A) r.a[k] = ell_load(a + e);
+                r.b[k] = ell_load(b + e);
+                r.c[k] = ell_load(c + e);
+            }
         }
+    }
+    template <bool A = true>
+    __device__ __forceinline__ Row row(int32_t i) const {
+        Row r;
+        r.i = i;
+        r.deg = __ldg(deg + i);
+        const int32_t s0 = __ldg(sbase + (i >> 5));
+        if (r.deg == 255) r.deg = __ldg(sbase + (i >> 5) + 1) - s0;  // (entries past its own: itself, zero)
+        r.p = (size_t)s0 * 32 + (i & 31);
+        load<A>(r.p, i, r.deg, 0, r.k[0]);
+        load<A>(r.p, i, r.deg, kChunk, r.k[1]);
+        return r;
+    }
+    // fn for the entries of a chunk; get(k, a): the recovery coefficients of
+    // the row's k-th entry where the chunk was loaded without them
+    template <typename Fn, typename Get>
+    __device__ __forceinline__ void chunk(const Chunk &r, int k0, Fn &&fn, Get &&get) const {
+#pragma unroll
+        for (int k = 0; k < kChunk; ++k) {
+            const int32_t j = ell_get(r.c[k].y);
+            const Ell2<T> a = get(k0 + k, r.a[k]);
+            if (chk_idx(j, n, 1u)) fn(j, a.x, a.y, r.b[k].x, r.b[k].y, r.c[k].x);
+        }
+    }
+    template <bool A = true, typename Fn, typename Get>
+    __device__ __forceinline__ void each_get(const Row &r, Fn &&fn, Get &&get) const {
+        chunk(r.k[0], 0, fn, get);
+        if (r.deg > kChunk) chunk(r.k[1], kChunk, fn, get);
+        for (int k = 2 * kChunk; k < r.deg; k += kChunk) {
+            Chunk c2;
+            load<A>(r.p, r.i, r.deg, k, c2);
+            chunk(c2, k, fn, get);
+        }
+    }
+    template <typename Fn>
+    __device__ __forceinline__ void each(const Row &r, Fn &&fn) const {
+        each_get(r, fn, [](int, Ell2<T> v) { return v; });
     }
     __device__ __forceinline__ int tag_of(int32_t i) const { return tag ? (int)tag[i] : 0; }
     // population storage: slot of node i, slots per population array
@@ -221,8 +361,10 @@ struct DevLattice {
     int32_t row0, gny;  // storage row y is row y + row0 of a lattice of gny rows
     T c[3][6][5];  // ax, ay, bxx, bxy, byy
 #ifdef __CUDACC__
+    using Row = int32_t;
+    __device__ __forceinline__ Row row(int32_t i) const { return i; }
     template <typename Fn>
-    __device__ __forceinline__ void for_each(int32_t i, Fn &&fn) const {
+    __device__ __forceinline__ void each(Row i, Fn &&fn) const {
         const int32_t y = i / nx, x = i - y * nx, gy = y + row0;
         const int kind = walls ? (gy == 0 ? 1 : (gy == gny - 1 ? 2 : 0)) : 0;
 #pragma unroll
@@ -329,14 +471,19 @@ struct felbm_mesh {
     felbm::Lattice3Info linfo3;
     felbm::StructuredInfo sinfo;
     // device arrays
-    int32_t *d_rowptr = nullptr, *d_col = nullptr, *d_perm = nullptr;
-    double *d_coef64 = nullptr;  // 5 * nnz, SoA: ax, ay, bxx, bxy, byy (kind 2: 9 * nnz, HostCSR3)
-    float *d_coef32 = nullptr;
+    int32_t *d_perm = nullptr;
+    // general meshes (kinds 0 and 2): rows in slices of 32 nodes, per
+    // precision {FP32, FP64} the entries of DevELL / DevELL3
+    int32_t *d_sbase = nullptr;
+    void *d_ell[2][4] = {};
+    uint8_t *d_deg = nullptr;  // neighbours of each node (kind 0)
     double *d_mass = nullptr;
     uint8_t *d_tag = nullptr;
-    // patches of the one-launch step of general triangle meshes (HostCSR)
-    int32_t *d_pnbase = nullptr, *d_pcount = nullptr, *d_pnode = nullptr, *d_prowbase = nullptr;
-    uint16_t *d_plcol = nullptr;
+    // patches of general triangle meshes (HostCSR), with the recovery
+    // coefficients a of their rows per precision {FP32, FP64}
+    int32_t *d_pnbase = nullptr, *d_pcount = nullptr, *d_pnode = nullptr, *d_pslice = nullptr, *d_psbase = nullptr;
+    uint16_t *d_pcol = nullptr;
+    void *d_pa[2] = {nullptr, nullptr};
     bool patch_step = false;
     int64_t device_bytes = 0;
 };
@@ -386,6 +533,12 @@ int prof_begin(felbm_state *s, int kind);
 // Shared helpers of the C ABI (felbm_api.cu) and its 3-D part (felbm_api3.cu).
 constexpr int kTotalsBlocks = 304;  // 2 x 152 SMs
 int cuda_status(cudaError_t e);
+// Upload `bytes` of host data to a new device array of mesh m (counted in
+// its device_bytes).
+cudaError_t mesh_upload(felbm_mesh *m, void **d, const void *host, size_t bytes);
+// Slices of 32 rows: sbase[s] is the first of slice s's rows of 32 entries,
+// as many as the longest of its CSR rows.
+std::vector<int32_t> ell_slices(int32_t n, const std::vector<int32_t> &rowptr);
 bool params_ok(const felbm_params *p);
 void mesh_free(felbm_mesh *m);
 void state_free(felbm_state *s);

@@ -115,44 +115,35 @@ __device__ __forceinline__ V2<T> pair_coef(int q, T ax, T ay, T hbxx, T hbxy, T 
     return vset(even + odd, even - odd);
 }
 
-// Streamed pairs of node i from the state f (pair layout, np = padded slot
-// count): psi* = psi - dt sum_{j != i} c_ij (psi_j - psi_i) for the 4 h
-// pairs and, with G, the 4 g pairs, one 8-byte load per pair and neighbour
-// and the neighbour's coefficients loaded once.
-template <typename T, bool G, typename Topo>
-__device__ __forceinline__ void stream_pairs(const Topo &m, const T *__restrict__ f, size_t np, int32_t i,
-                                             T dt, V2<T> *hp, V2<T> *gp) {
-    const V2<T> *hb = reinterpret_cast<const V2<T> *>(f + np);
-    const V2<T> *gb = reinterpret_cast<const V2<T> *>(f + 10 * np);
+// Streamed pairs of node i of one distribution (f: its rest values, pair q
+// at f + np + 2 np q, np = padded slot count): psi* = psi - dt sum_{j != i}
+// c_ij (psi_j - psi_i), one 8-byte load per pair and neighbour.  each(fn)
+// calls fn(j, ax, ay, bxx, bxy, byy) for the node's neighbours.
+template <typename T, typename Topo, typename Each>
+__device__ __forceinline__ void stream_pairs(const Topo &m, const T *f, size_t np, int32_t i, T dt, V2<T> *out,
+                                             Each &&each) {
+    const V2<T> *pb = reinterpret_cast<const V2<T> *>(f + np);
     const size_t si = m.slot(i);
     const V2<T> m1 = vset(T(-1), T(-1));
-    V2<T> hs[4], ha[4], gs[4], ga[4];
+    V2<T> own[4], acc[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        hs[q] = hb[q * np + si];
-        ha[q] = vset(T(0), T(0));
-        if (G) {
-            gs[q] = gb[q * np + si];
-            ga[q] = vset(T(0), T(0));
-        }
+        own[q] = pb[q * np + si];
+        acc[q] = vset(T(0), T(0));
     }
     const T hdt = T(0.5) * dt;
-    m.for_each(i, [&](int32_t j, T ax, T ay, T bxx, T bxy, T byy) {
+    each([&](int32_t j, T ax, T ay, T bxx, T bxy, T byy) {
         const size_t sj = m.slot(j);
         const T hbxx = hdt * bxx, hbxy = hdt * bxy, hbyy = hdt * byy;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const V2<T> c = pair_coef<T>(q, ax, ay, hbxx, hbxy, hbyy);
-            ha[q] = vfma(c, vfma(hs[q], m1, __ldg(hb + q * np + sj)), ha[q]);
-            if (G) ga[q] = vfma(c, vfma(gs[q], m1, __ldg(gb + q * np + sj)), ga[q]);
+            acc[q] = vfma(c, vfma(own[q], m1, pb[q * np + sj]), acc[q]);
         }
     });
     const V2<T> mdt = vset(-dt, -dt);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        hp[q] = vfma(mdt, ha[q], hs[q]);
-        if (G) gp[q] = vfma(mdt, ga[q], gs[q]);
-    }
+    for (int q = 0; q < 4; ++q) out[q] = vfma(mdt, acc[q], own[q]);
 }
 
 // Populations of a node by direction from its rest value and 4 pairs.
@@ -176,20 +167,23 @@ __device__ __forceinline__ void bounce_back(int k, T *psi) {
         if (kEx(a) * nx + kEy(a) * ny > 0) psi[a] = psi[kOpp(a)];
 }
 
-template <typename T, typename Topo>
-__global__ void __launch_bounds__(256) k_rho(Topo m, const T *__restrict__ f, T dt,
-                                             T *__restrict__ rho, T *__restrict__ hs) {
+// ONE: the mesh's blocks are all resident at once (see kOneWave); they may
+// then have more registers, for more gathers in flight.
+template <typename T, typename Topo, bool ONE>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (ONE ? 4 : 5) : 2)
+    k_rho(const __grid_constant__ Topo m, const T *f, T dt, T *rho, T *hs) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.n) return;
     const size_t np = pad4(m.slots());
+    const auto row = m.row(i);
+    const int k = m.tag_of(i);
+    pdl_wait();
+    pdl_trigger();
     V2<T> hp[4];
-    stream_pairs<T, false>(m, f, np, i, dt, hp, hp);
+    stream_pairs<T>(m, f, np, i, dt, hp, [&](auto &&fn) { m.each(row, fn); });
     T h[9];
     unpack_pairs<T>(f[m.slot(i)], hp, h);
-    {
-        const int k = m.tag_of(i);
-        if (k) bounce_back<T>(k, h);
-    }
+    if (k) bounce_back<T>(k, h);
     T r = T(0);
 #pragma unroll
     for (int a = 0; a < 9; ++a) r += h[a];
@@ -201,27 +195,31 @@ __global__ void __launch_bounds__(256) k_rho(Topo m, const T *__restrict__ f, T 
     hs[si] = h[0];
 }
 
+// One neighbour's part of a recovered gradient (d: difference of the field).
+template <typename T>
+__device__ __forceinline__ void grad_edge(T ax, T ay, T d, T &gx, T &gy) {
+    gx = fma(ax, d, gx);
+    gy = fma(ay, d, gy);
+}
+
 // Recovered gradient of a scalar field.
 template <typename T, typename Topo>
-__device__ __forceinline__ void recover(const Topo &m, const T *__restrict__ f, int32_t i,
-                                        T &gx, T &gy) {
+__device__ __forceinline__ void recover(const Topo &m, const typename Topo::Row &row, const T *f,
+                                        int32_t i, T &gx, T &gy) {
     const T fi = f[i];
-    T sx = T(0), sy = T(0);
-    m.for_each(i, [&](int32_t j, T ax, T ay, T, T, T) {
-        const T d = __ldg(f + j) - fi;
-        sx += ax * d;
-        sy += ay * d;
-    });
-    gx = sx;
-    gy = sy;
+    gx = gy = T(0);
+    m.each(row, [&](int32_t j, T ax, T ay, T, T, T) { grad_edge<T>(ax, ay, f[j] - fi, gx, gy); });
 }
 
 template <typename T, typename Topo>
-__global__ void __launch_bounds__(256) k_grad(Topo m, Fields<T> F) {
+__global__ void __launch_bounds__(256) k_grad(const __grid_constant__ Topo m, Fields<T> F) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.n) return;
+    const auto row = m.row(i);
+    pdl_wait();
+    pdl_trigger();
     T gx, gy;
-    recover(m, F.rho, i, gx, gy);
+    recover(m, row, F.rho, i, gx, gy);
     F.drx[i] = gx;
     F.dry[i] = gy;
 }
@@ -238,21 +236,35 @@ __device__ __forceinline__ T mu_bulk(const Phys<T> &P, T r) {
 // (the printed form d_i(|grad rho|^2) - d_j(d_i rho d_j rho) with the
 // identical (d_i rho)^2 contributions cancelled, R linear);
 // mu = 4 beta (rho - rho_v)(rho - rho_l)(rho - (rho_v + rho_l)/2) - kappa lap rho.
+// One neighbour's part of K / kappa, with the differences of the gradient
+// products in product form (no cancellation between two squares of nearly
+// equal size).
+template <typename T>
+__device__ __forceinline__ void stress_edge(T ax, T ay, T gxi, T gyi, T gxj, T gyj, T &kx, T &ky) {
+    const T ddx = gxj - gxi, ddy = gyj - gyi;
+    const T dxx = ddx * (gxj + gxi), dxy = fma(gxj, ddy, gyi * ddx), dyy = ddy * (gyj + gyi);
+    kx = fma(ax, dyy, fma(-ay, dxy, kx));
+    ky = fma(ay, dxx, fma(-ax, dxy, ky));
+}
+// One neighbour's part of lap rho.
+template <typename T>
+__device__ __forceinline__ void lap_edge(T ax, T ay, T gxi, T gyi, T gxj, T gyj, T &lap) {
+    lap = fma(ax, gxj - gxi, fma(ay, gyj - gyi, lap));
+}
+
 template <typename T, typename Topo>
-__global__ void __launch_bounds__(256) k_mu(Topo m, Fields<T> F, Phys<T> P) {
+__global__ void __launch_bounds__(256) k_mu(const __grid_constant__ Topo m, Fields<T> F, Phys<T> P) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.n) return;
+    const auto row = m.row(i);
+    pdl_wait();
+    pdl_trigger();
     const T gxi = F.drx[i], gyi = F.dry[i];
     T lap = T(0), kx = T(0), ky = T(0);
-    m.for_each(i, [&](int32_t j, T ax, T ay, T, T, T) {
-        const T gxj = __ldg(F.drx + j), gyj = __ldg(F.dry + j);
-        lap += ax * (gxj - gxi) + ay * (gyj - gyi);
-        // differences of the gradient products in product form (no
-        // cancellation between two squares of nearly equal size)
-        const T ddx = gxj - gxi, ddy = gyj - gyi;
-        const T dxx = ddx * (gxj + gxi), dxy = gxj * ddy + gyi * ddx, dyy = ddy * (gyj + gyi);
-        kx += ax * dyy - ay * dxy;
-        ky += ay * dxx - ax * dxy;
+    m.each(row, [&](int32_t j, T ax, T ay, T, T, T) {
+        const T gxj = F.drx[j], gyj = F.dry[j];
+        lap_edge<T>(ax, ay, gxi, gyi, gxj, gyj, lap);
+        stress_edge<T>(ax, ay, gxi, gyi, gxj, gyj, kx, ky);
     });
     F.mu[i] = mu_bulk<T>(P, F.rho[i]) - P.kappa * lap;
     F.kx[i] = P.kappa * kx;
@@ -265,20 +277,20 @@ __global__ void __launch_bounds__(256) k_mu(Topo m, Fields<T> F, Phys<T> P) {
 // FP64 and subtracted from the bulk term in FP64, rounded once.  K is formed
 // as in k_mu, from the same coefficients rounded to FP32.
 template <typename Topo64>
-__global__ void __launch_bounds__(256) k_mu_lap64(Topo64 m, Fields<float> F, Phys<float> P, double kappa) {
+__global__ void __launch_bounds__(256) k_mu_lap64(const __grid_constant__ Topo64 m, Fields<float> F, Phys<float> P,
+                                                  double kappa) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.n) return;
+    const auto row = m.row(i);
+    pdl_wait();
+    pdl_trigger();
     const float gxi = F.drx[i], gyi = F.dry[i];
     double lap = 0.0;
     float kx = 0.f, ky = 0.f;
-    m.for_each(i, [&](int32_t j, double ax, double ay, double, double, double) {
-        const float gxj = __ldg(F.drx + j), gyj = __ldg(F.dry + j);
-        lap += ax * ((double)gxj - (double)gxi) + ay * ((double)gyj - (double)gyi);
-        const float fax = (float)ax, fay = (float)ay;
-        const float ddx = gxj - gxi, ddy = gyj - gyi;
-        const float dxx = ddx * (gxj + gxi), dxy = gxj * ddy + gyi * ddx, dyy = ddy * (gyj + gyi);
-        kx += fax * dyy - fay * dxy;
-        ky += fay * dxx - fax * dxy;
+    m.each(row, [&](int32_t j, double ax, double ay, double, double, double) {
+        const float gxj = F.drx[j], gyj = F.dry[j];
+        lap_edge<double>(ax, ay, gxi, gyi, gxj, gyj, lap);
+        stress_edge<float>((float)ax, (float)ay, gxi, gyi, gxj, gyj, kx, ky);
     });
     F.mu[i] = (float)((double)mu_bulk<float>(P, F.rho[i]) - kappa * lap);
     F.kx[i] = P.kappa * kx;
@@ -444,35 +456,22 @@ struct CollideArgs {
     int *flag;
 };
 
+// Collision and write of one node of a general mesh from its streamed,
+// bounced-back g and the h* of k_rho.
 template <typename T, typename Topo>
-__global__ void __launch_bounds__(256) k_collide(CollideArgs<T, Topo> A) {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    const Topo &m = A.m;
-    if (i >= m.n) return;
-    const size_t n = (size_t)m.n;
-    T dmx, dmy;
-    recover(m, A.F.mu, i, dmx, dmy);
-    const size_t np = pad4(m.slots()), si = m.slot(i);
-    T hs[9], gs[9];
+__device__ __forceinline__ void collide_write(const CollideArgs<T, Topo> &A, int32_t i, size_t np, const T *gs, T r,
+                                              T drx, T dry, T dmx, T dmy, T kx, T ky) {
+    const size_t n = (size_t)A.m.n, si = A.m.slot(i);
+    T hs[9];
     {
-        // g streamed here (the h code on the g half of the state); h* was
-        // streamed and bounced back by k_rho
-        V2<T> gp[4], hp[4];
-        stream_pairs<T, false>(m, A.fin + 9 * np, np, i, A.P.dt, gp, gp);
-        unpack_pairs<T>(A.fin[9 * np + si], gp, gs);
+        V2<T> hp[4];
         const V2<T> *hsb = reinterpret_cast<const V2<T> *>(A.F.hs + np);
 #pragma unroll
         for (int q = 0; q < 4; ++q) hp[q] = hsb[q * np + si];
         unpack_pairs<T>(A.F.hs[si], hp, hs);
     }
-    {
-        const int k = m.tag_of(i);
-        if (k) bounce_back<T>(k, gs);
-    }
-    const T r = A.F.rho[i];
     T hout[9], gout[9], ux, uy, p;
-    collide_node<T>(A.P, hs, gs, r, A.F.drx[i], A.F.dry[i], dmx, dmy, A.F.kx[i], A.F.ky[i], hout,
-                    gout, ux, uy, p);
+    collide_node<T>(A.P, hs, gs, r, drx, dry, dmx, dmy, kx, ky, hout, gout, ux, uy, p);
     V2<T> *hb = reinterpret_cast<V2<T> *>(A.fout + np);
     V2<T> *gb = reinterpret_cast<V2<T> *>(A.fout + 10 * np);
 #pragma unroll
@@ -491,16 +490,39 @@ __global__ void __launch_bounds__(256) k_collide(CollideArgs<T, Topo> A) {
     }
 }
 
+template <typename T, typename Topo>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 2) k_collide(const __grid_constant__ CollideArgs<T, Topo> A) {
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    const Topo &m = A.m;
+    if (i >= m.n) return;
+    const size_t np = pad4(m.slots());
+    const auto row = m.row(i);
+    const int k = m.tag_of(i);
+    pdl_wait();
+    pdl_trigger();
+    T dmx, dmy, gs[9];
+    {
+        // g streamed here (the h code on the g half of the state); h* was
+        // streamed and bounced back by k_rho
+        V2<T> gp[4];
+        stream_pairs<T>(m, A.fin + 9 * np, np, i, A.P.dt, gp, [&](auto &&fn) { m.each(row, fn); });
+        unpack_pairs<T>(A.fin[9 * np + m.slot(i)], gp, gs);
+        if (k) bounce_back<T>(k, gs);
+    }
+    recover(m, row, A.F.mu, i, dmx, dmy);
+    collide_write<T>(A, i, np, gs, A.F.rho[i], A.F.drx[i], A.F.dry[i], dmx, dmy, A.F.kx[i], A.F.ky[i]);
+}
+
 // Initial state: post-collision distributions are the equilibria of
 // (rho0, u0, p0); stored value psibar = eq + S (Omega(eq) = 0).
 template <typename T, typename Topo>
-__global__ void __launch_bounds__(256) k_init(Topo m, T *__restrict__ fout, Fields<T> F,
+__global__ void __launch_bounds__(256) k_init(const __grid_constant__ Topo m, T *__restrict__ fout, Fields<T> F,
                                               Phys<T> P, const T *__restrict__ mom) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.n) return;
     const size_t n = (size_t)m.n;
     T dmx, dmy;
-    recover(m, F.mu, i, dmx, dmy);
+    recover(m, m.row(i), F.mu, i, dmx, dmy);
     const T r = mom[i], ux = mom[n + i], uy = mom[2 * n + i], p = mom[3 * n + i];
     const T drx = F.drx[i], dry = F.dry[i], kx = F.kx[i], ky = F.ky[i];
     const T hdt = T(0.5) * P.dt;

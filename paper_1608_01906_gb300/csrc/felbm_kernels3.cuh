@@ -1,5 +1,5 @@
 // Device kernels of one FE-LBM time step on tetrahedral meshes (D3Q19, the
-// paper's own setting), on two topologies: the general CSR (DevCSR3) and the
+// paper's own setting), on two topologies: general rows (DevELL3) and the
 // Kuhn-split cube lattice (DevLattice3).  Same four dependent passes as the
 // two-dimensional general path (felbm_kernels.cuh):
 //   k_rho3      Taylor-Galerkin streaming of the 19 h populations (Sec.
@@ -63,31 +63,37 @@ __device__ __forceinline__ T mu_bulk3(const Phys3<T> &P, T r) {
     return T(4) * P.beta * (r - P.rho_v) * (r - P.rho_l) * (r - T(0.5) * (P.rho_v + P.rho_l));
 }
 
-// General tetrahedral mesh: CSR in reverse Cuthill-McKee order with the
-// coefficient arrays of HostCSR3 (a: 3, b: 6 symmetric components).
 // Both topologies give, for node i, the neighbours j with their
 // coefficients: for_each<K>(i, fn(j, a)) with a = (a_x, a_y, a_z) at least,
 // for_each_pair<K>(i, dt/2, fn(j, c)) with c[q] = (e.a + dt/2 e.b.e) for the
 // pair q = (2q+1, 2q+2) as (first, second) = (even + odd, even - odd) parts.
 // K >= 0 promises that node i is of z-layer kind K (lattice only; -1 = any).
+//
+// General tetrahedral mesh, reverse Cuthill-McKee order: rows in slices of
+// 32 nodes (see DevELL), per entry {a_x, a_y, a_z, neighbour}, {b_xx, b_xy,
+// b_xz, b_yy} and {b_yz, b_zz}.
 template <typename T>
-struct DevCSR3 {
+struct DevELL3 {
     static constexpr bool kLattice = false;
     int32_t n;
-    const int32_t *rowptr;
-    const int32_t *col;
-    const T *c[9];       // ax, ay, az, bxx, bxy, bxz, byy, byz, bzz (nnz each)
+    const int32_t *sbase;
+    const Ell4<T> *a, *b;
+    const Ell2<T> *c;
     const uint8_t *tag;  // nullptr if no walls
 #ifdef __CUDACC__
     template <int K, typename Fn>
     __device__ __forceinline__ void for_each(int32_t i, Fn &&fn) const {
-        const int32_t p1 = __ldg(rowptr + i + 1);
-        for (int32_t p = __ldg(rowptr + i); p < p1; ++p) {
-            const int32_t j = __ldg(col + p);
+        const int32_t r0 = __ldg(sbase + (i >> 5)), r1 = __ldg(sbase + (i >> 5) + 1);
+        const size_t p = (size_t)r0 * 32 + (i & 31);
+        const Ell4<T> *pa = a + p, *pb = b + p;
+        const Ell2<T> *pc = c + p;
+#pragma unroll 4
+        for (int32_t k = 0; k < r1 - r0; ++k) {
+            const Ell4<T> v = ell_load(pa + 32 * k), w = ell_load(pb + 32 * k);
+            const Ell2<T> z = ell_load(pc + 32 * k);
+            const int32_t j = ell_get(v.w);
             if (!chk_idx(j, n, 1u)) continue;
-            T cf[9];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) cf[k] = __ldg(c[k] + p);
+            const T cf[9] = {v.x, v.y, v.z, w.x, w.y, w.z, w.w, z.x, z.y};
             fn(j, cf);
         }
     }

@@ -182,15 +182,13 @@ static std::vector<int32_t> patch_order(const double *xy, int32_t N, const doubl
     return order;
 }
 
-// Rings of every patch over the CSR in internal (patch-major) order.
+// Rings of every patch over the CSR in internal (patch-major) order, and
+// the sliced rows of its rings <= 2.
 static void build_patches(HostCSR &H) {
     const int32_t N = H.n, np = (N + kPatch - 1) / kPatch;
     H.pnbase.assign((size_t)np + 1, 0);
     H.pcount.assign((size_t)4 * np, 0);
-    H.pnode.clear();
-    H.prowbase.clear();
-    H.plcol.clear();
-    H.rmax = H.r1max = H.r2max = H.r3max = 0;
+    H.pslice.assign((size_t)np, 0);
     std::vector<int32_t> stamp((size_t)N, -1), loc((size_t)N, 0);
     std::vector<int32_t> reg;
     for (int32_t p = 0; p < np; ++p) {
@@ -200,10 +198,9 @@ static void build_patches(HostCSR &H) {
             loc[i] = (int32_t)reg.size();
             reg.push_back(i);
         }
-        int32_t cnt[4];
+        int32_t cnt[4] = {(int32_t)reg.size(), 0, 0, 0};
         size_t ring0 = 0;
-        for (int ring = 1; ring <= 4; ++ring) {
-            cnt[ring - 1] = (int32_t)reg.size();
+        for (int ring = 1; ring <= 3; ++ring) {
             const size_t ring1 = reg.size();
             for (size_t k = ring0; k < ring1; ++k)
                 for (int32_t e = H.rowptr[reg[k]]; e < H.rowptr[reg[k] + 1]; ++e) {
@@ -215,28 +212,37 @@ static void build_patches(HostCSR &H) {
                     }
                 }
             ring0 = ring1;
+            cnt[ring] = (int32_t)reg.size();
         }
-        if (reg.size() > 65535) {  // region indices are 16-bit: no patch step
-            H.pnbase.clear();
-            H.pcount.clear();
-            H.pnode.clear();
-            H.prowbase.clear();
-            H.plcol.clear();
+        const int32_t slices = (cnt[2] + 31) / 32;
+        // region indices are 16-bit, entry offsets 32-bit: else no patch step
+        if (reg.size() > 65535 || H.pcsr.size() > (size_t)0x60000000) {
+            for (auto *v : {&H.pnbase, &H.pcount, &H.pnode, &H.pslice, &H.psbase, &H.pcsr}) v->clear();
+            H.pcol.clear();
             return;
         }
         for (int r = 0; r < 4; ++r) H.pcount[4 * p + r] = cnt[r];
         H.pnbase[p + 1] = H.pnbase[p] + (int32_t)reg.size();
-        for (size_t r = 0; r < reg.size(); ++r) {
-            H.pnode.push_back(reg[r]);
-            if ((int32_t)r < cnt[3]) {
-                H.prowbase.push_back((int32_t)H.plcol.size());
-                for (int32_t e = H.rowptr[reg[r]]; e < H.rowptr[reg[r] + 1]; ++e)
-                    H.plcol.push_back((uint16_t)loc[H.col[e]]);
-            } else {
-                H.prowbase.push_back(-1);
-            }
+        H.pnode.insert(H.pnode.end(), reg.begin(), reg.end());
+        H.pslice[p] = (int32_t)H.psbase.size();
+        const size_t first = H.pcsr.size() / 32;
+        for (int32_t s = 0; s < slices; ++s) {
+            H.psbase.push_back((int32_t)(H.pcsr.size() / 32));
+            int32_t w = 0;
+            for (int32_t r = 32 * s; r < std::min(cnt[2], 32 * (s + 1)); ++r)
+                w = std::max(w, H.rowptr[reg[r] + 1] - H.rowptr[reg[r]]);
+            for (int32_t k = 0; k < w; ++k)
+                for (int32_t r = 32 * s; r < 32 * (s + 1); ++r) {
+                    const int32_t g = reg[std::min(r, cnt[2] - 1)];
+                    const int32_t e = H.rowptr[g] + k;
+                    const bool in = r < cnt[2] && e < H.rowptr[g + 1];
+                    H.pcsr.push_back(in ? e : -1);
+                    H.pcol.push_back((uint16_t)(in ? loc[H.col[e]] : std::min(r, cnt[2] - 1)));
+                }
         }
-        H.rmax = std::max(H.rmax, (int32_t)reg.size());
+        H.psbase.push_back((int32_t)(H.pcsr.size() / 32));
+        H.pemax = std::max(H.pemax, (int32_t)(H.pcsr.size() / 32 - first));
+        H.psmax = std::max(H.psmax, slices);
         H.r1max = std::max(H.r1max, cnt[1]);
         H.r2max = std::max(H.r2max, cnt[2]);
         H.r3max = std::max(H.r3max, cnt[3]);
