@@ -146,25 +146,17 @@ __device__ __forceinline__ void stream_pairs(const Topo &m, const T *f, size_t n
     for (int q = 0; q < 4; ++q) out[q] = vfma(mdt, acc[q], own[q]);
 }
 
-// Populations of a node by direction from its rest value and 4 pairs.
-template <typename T>
-__device__ __forceinline__ void unpack_pairs(T rest, const V2<T> *p, T *psi) {
-    psi[0] = rest;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        psi[pair_dir(q, 0)] = p[q].x;
-        psi[pair_dir(q, 1)] = p[q].y;
-    }
-}
-
 // Bounce-back at a wall node with inward normal e_k: every population with
-// e_a . e_k > 0 takes the value of its opposite.  psi holds 9 populations.
+// e_a . e_k > 0 takes the value of its opposite.
 template <typename T>
-__device__ __forceinline__ void bounce_back(int k, T *psi) {
+__device__ __forceinline__ void bounce_pairs(int k, V2<T> *p) {
     const int nx = kEx(k), ny = kEy(k);
 #pragma unroll
-    for (int a = 1; a < 9; ++a)
-        if (kEx(a) * nx + kEy(a) * ny > 0) psi[a] = psi[kOpp(a)];
+    for (int q = 0; q < 4; ++q) {
+        const int a = pair_dir(q, 0), d = kEx(a) * nx + kEy(a) * ny;
+        if (d > 0) p[q].x = p[q].y;
+        if (d < 0) p[q].y = p[q].x;
+    }
 }
 
 // ONE: the mesh's blocks are all resident at once (see kOneWave); they may
@@ -181,18 +173,14 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (ONE ? 4 : 5) : 2)
     pdl_trigger();
     V2<T> hp[4];
     stream_pairs<T>(m, f, np, i, dt, hp, [&](auto &&fn) { m.each(row, fn); });
-    T h[9];
-    unpack_pairs<T>(f[m.slot(i)], hp, h);
-    if (k) bounce_back<T>(k, h);
-    T r = T(0);
-#pragma unroll
-    for (int a = 0; a < 9; ++a) r += h[a];
-    rho[i] = r;
     const size_t si = m.slot(i);
+    const T h0 = f[si];
+    if (k) bounce_pairs<T>(k, hp);
+    rho[i] = ((h0 + (hp[0].x + hp[0].y)) + (hp[1].x + hp[1].y)) + ((hp[2].x + hp[2].y) + (hp[3].x + hp[3].y));
     V2<T> *hb = reinterpret_cast<V2<T> *>(hs + np);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) hb[q * np + si] = vset(h[pair_dir(q, 0)], h[pair_dir(q, 1)]);
-    hs[si] = h[0];
+    for (int q = 0; q < 4; ++q) hb[q * np + si] = hp[q];
+    hs[si] = h0;
 }
 
 // One neighbour's part of a recovered gradient (d: difference of the field).
@@ -301,19 +289,35 @@ __global__ void __launch_bounds__(256) k_mu_lap64(const __grid_constant__ Topo64
 // keep the streamed populations outside registers:
 //   collide_prep  moments (Eqs. velocity, pressure), tau, and the per-node
 //                 scalars of the equilibria and sources;
-//   collide_pop   the update of population a.
+//   collide_pair  the update of a pair of opposite directions.
 // With eq and source S of the node, the post-streaming collision
 //   psi = psi* + 2tau/(2tau+1) (-(psi* - eq)/(2tau) + S)
 // followed by the pre-streaming collision of the next step
 //   psibar = psi + (-(psi - eq)/(2tau) + S)
 // equals psibar = eq + S + w (psi* - eq + S), w = (2tau - 1)/(2tau + 1),
-// evaluated as psibar = psi* + (1 - w)(eq - psi*) + (1 + w) S with
-// eq - psi* = fma(rho, w_a, -psi*) + rho (Gamma - w_a): every rounding then
-// falls on the small collision increment instead of on O(w_a rho) terms
+// evaluated as psibar = psi* + (1 - w)(eq - psi*) + (1 + w) S: every rounding
+// then falls on the small collision increment instead of on O(w_a rho) terms
 // (in FP32 the other order repeats the same O(ulp(rho)) error every step).
+// With q = e.u + 3/2 (e.u)^2 - u.u/2 (so that Gamma_a - w_a = 3 w_a q and
+// 3 Gamma_a = 3 w_a (1 + 3 q)) and the forces scaled by (1 + w) dt/2 once per
+// node, the increments are
+//   h: -(1-w) (h* - rho w_a) + 3 w_a [c + q (m + 3 c)],
+//      c = (e-u).X, X = c_s^2 grad rho - rho grad mu, m = (1-w) rho;
+//   g: -(1-w) (g* - 3 w_a p) + 3 w_a [k + b + q (m + d + 3 k)],
+//      k = (e-u).K, d = (e-u).grad rho, b the exact-difference body force
+//      (1+w) rho/2 [e.du + e.du (3 e.u + 3/2 e.du) - du.(2u + du)/2]:
+// two products per population with sums that are the node's but for the sign
+// of their odd part, 23 packed operations for a pair against 56 when each
+// term was formed by itself.
 template <typename T>
 struct CollidePrep {
-    T r, ux, uy, p, omw, opw, hdt, Xx, Xy, uX, uD, uK, uu, dux, duy, udu, drx, dry, kx, ky;
+    T r, ux, uy, p;
+    T nr, np, nomw;   // -rho, -p, -(1 - w)
+    T nhuu;           // -u.u/2
+    T Xx, Xy, hA, hZ; // X (scaled); even parts m - 3 u.X and -u.X
+    T Vx, Vy, gA;     // grad rho + 3 K (scaled); even part m - u.V
+    T Bx, By, gZ;     // K + G; even part -u.K - (1+w) rho/4 du.(2u + du)
+    T Gx, Gy, dux, duy;  // (1+w) rho/2 du, and du
 };
 
 // Correctly rounded reciprocal (the same value as T(1) / x).
@@ -339,76 +343,89 @@ __device__ __forceinline__ CollidePrep<T> collide_prep(const Phys<T> &P, T sg, T
                                                        T drx, T dry, T dmx, T dmy, T kx, T ky) {
     constexpr T cs2 = T(1) / T(3);
     CollidePrep<T> c;
-    c.hdt = T(0.5) * P.dt;
+    const T hdt = T(0.5) * P.dt;
     const T inv_r = recip_rn(r);
     c.r = r;
-    c.ux = (mx + c.hdt * kx + c.hdt * r * P.gx) * inv_r;
-    c.uy = (my + c.hdt * ky + c.hdt * r * P.gy) * inv_r;
+    c.ux = (mx + hdt * kx + hdt * r * P.gx) * inv_r;
+    c.uy = (my + hdt * ky + hdt * r * P.gy) * inv_r;
     // p = c_s^2 (...) as a division by 3: a rounded 1/3 would be a gain on p
     // every step (see kW3)
-    c.p = div3(sg + c.hdt * (c.ux * drx + c.uy * dry));
+    c.p = div3(sg + hdt * (c.ux * drx + c.uy * dry));
     T C = (r - P.rho_v) * P.inv_drho;
     C = C < T(0) ? T(0) : (C > T(1) ? T(1) : C);
     // 1/tau = C/tau_l + (1-C)/tau_v; w = (2 tau - 1)/(2 tau + 1) gives, with
     // s = 1/tau, 1 - w = 2 s/(2 + s) and 1 + w = 4/(2 + s): one reciprocal
     const T s = C * P.inv_tau_l + (T(1) - C) * P.inv_tau_v;
     const T d = recip_rn(T(2) + s);
-    c.omw = T(2) * s * d;  // 1 - w
-    c.opw = T(4) * d;      // 1 + w
-    c.Xx = cs2 * drx - r * dmx;  // F: c_s^2 grad rho - rho grad mu
-    c.Xy = cs2 * dry - r * dmy;
-    c.uX = c.ux * c.Xx + c.uy * c.Xy;
-    c.uD = c.ux * drx + c.uy * dry;
-    c.uK = c.ux * kx + c.uy * ky;
-    c.uu = c.ux * c.ux + c.uy * c.uy;
+    const T omw = T(2) * s * d, opw = T(4) * d;
+    const T f = opw * hdt, m = omw * r;
+    c.nr = -r;
+    c.np = -c.p;
+    c.nomw = -omw;
+    c.nhuu = T(-0.5) * (c.ux * c.ux + c.uy * c.uy);
+    c.Xx = f * (cs2 * drx - r * dmx);
+    c.Xy = f * (cs2 * dry - r * dmy);
+    const T uX = c.ux * c.Xx + c.uy * c.Xy;
+    c.hZ = -uX;
+    c.hA = fma(T(-3), uX, m);
+    const T Kx = f * kx, Ky = f * ky;
+    c.Vx = fma(T(3), Kx, f * drx);
+    c.Vy = fma(T(3), Ky, f * dry);
+    c.gA = m - (c.ux * c.Vx + c.uy * c.Vy);
     c.dux = P.gx * P.dt;  // exact-difference du = g dt
     c.duy = P.gy * P.dt;
-    c.udu = c.dux * (T(2) * c.ux + c.dux) + c.duy * (T(2) * c.uy + c.duy);
-    c.drx = drx;
-    c.dry = dry;
-    c.kx = kx;
-    c.ky = ky;
+    const T hr = T(0.5) * opw * r;
+    c.Gx = hr * c.dux;
+    c.Gy = hr * c.duy;
+    c.Bx = Kx + c.Gx;
+    c.By = Ky + c.Gy;
+    c.gZ = -(c.ux * Kx + c.uy * Ky) - (c.Gx * (c.ux + T(0.5) * c.dux) + c.Gy * (c.uy + T(0.5) * c.duy));
     return c;
 }
 
-template <typename T, int A>
-__device__ __forceinline__ void collide_pop(const CollidePrep<T> &c, T hs, T gs, T &hout, T &gout) {
-    constexpr int ex = kEx(A), ey = kEy(A);
-    constexpr T wa = kW<T>(A), w3 = kW3<T>(A);
-    const T eu = T(ex) * c.ux + T(ey) * c.uy;
-    // Gamma - w formed directly: forming Gamma ~ w first and subtracting w
-    // would cancel away the momentum part rho w 3 e.u in FP32.
-    const T gmw = w3 * (eu + T(1.5) * eu * eu - T(0.5) * c.uu);
-    const T gam3 = w3 + T(3) * gmw;  // 3 Gamma
-    const T eX = T(ex) * c.Xx + T(ey) * c.Xy;
-    const T eD = T(ex) * c.drx + T(ey) * c.dry;
-    const T eK = T(ex) * c.kx + T(ey) * c.ky;
-    const T edu = T(ex) * c.dux + T(ey) * c.duy;
-    const T Fa = c.hdt * (eX - c.uX) * gam3;
-    const T Ga = c.hdt * (eD - c.uD) * gmw + c.hdt * (eK - c.uK) * gam3;
-    // 1/2 [g_eq(u + du) - g_eq(u)] = rho/2 [Gamma(u + du) - Gamma(u)]
-    const T Ba = T(0.5) * c.r * w3 * (edu + T(1.5) * edu * (T(2) * eu + edu) - T(0.5) * c.udu);
-    const T Sg = Ga + Ba;
-    const T dh = fma(c.r, wa, -hs) + c.r * gmw;  // h_eq - h*
-    const T dg = fma(w3, c.p, -gs) + c.r * gmw;  // g_eq - g*
-    hout = hs + (c.omw * dh + c.opw * Fa);
-    gout = gs + (c.omw * dg + c.opw * Sg);
+// e.v for a direction known at compile time (no product)
+template <int EX, int EY, typename T>
+__device__ __forceinline__ T dir_dot(T x, T y) {
+    if (EX == 0) return EY > 0 ? y : -y;
+    if (EY == 0) return EX > 0 ? x : -x;
+    return (EX > 0 ? x : -x) + (EY > 0 ? y : -y);
 }
 
+// Collision of the opposite pair Q = (a, abar) of one node: e_abar = -e_a
+// and w_abar = w_a, so the odd parts flip sign between the two lanes and the
+// even parts are shared; the two lanes run in packed two-wide arithmetic.
+// ds takes the pair's h increments.
+template <typename T, int Q>
+__device__ __forceinline__ void collide_pair(const CollidePrep<T> &c, V2<T> hs, V2<T> gs, V2<T> &ho, V2<T> &go,
+                                             V2<T> &ds) {
+    constexpr int A = pair_dir(Q, 0), ex = kEx(A), ey = kEy(A);
+    constexpr T wa = kW<T>(A), w3 = kW3<T>(A);
+    const T eu = dir_dot<ex, ey>(c.ux, c.uy), eX = dir_dot<ex, ey>(c.Xx, c.Xy);
+    const T eV = dir_dot<ex, ey>(c.Vx, c.Vy), eB = dir_dot<ex, ey>(c.Bx, c.By);
+    const T eG = dir_dot<ex, ey>(c.Gx, c.Gy), ed = dir_dot<ex, ey>(c.dux, c.duy);
+    const T qe = fma(T(1.5) * eu, eu, c.nhuu), eA = T(3) * eX;
+    const T ge = fma(eG, fma(T(1.5), ed, T(3) * eu), c.gZ);
+    const V2<T> q = vset(qe + eu, qe - eu);
+    const V2<T> hz = vfma(q, vset(c.hA + eA, c.hA - eA), vset(c.hZ + eX, c.hZ - eX));
+    const V2<T> gz = vfma(q, vset(c.gA + eV, c.gA - eV), vset(ge + eB, ge - eB));
+    const V2<T> w32 = vset(w3, w3), nomw = vset(c.nomw, c.nomw);
+    const V2<T> hd = vfma(nomw, vfma(vset(c.nr, c.nr), vset(wa, wa), hs), vmul(w32, hz));
+    const V2<T> gd = vfma(nomw, vfma(vset(c.np, c.np), w32, gs), vmul(w32, gz));
+    ho = vadd(hs, hd);
+    go = vadd(gs, gd);
+    ds = vadd(ds, vfma(hs, vset(T(-1), T(-1)), ho));
+}
+
+// The same for the rest population; its h also takes the sum of the node's
+// h increments (zero in exact arithmetic; ds those of the pairs): the
+// collision then keeps the node's mass to one rounding instead of
+// accumulating the rounding of the nine source terms every step.
 template <typename T>
-__device__ __forceinline__ void collide_pop_rt(const CollidePrep<T> &c, int a, T hs, T gs, T &ho,
-                                               T &go) {
-    switch (a) {
-        case 0: collide_pop<T, 0>(c, hs, gs, ho, go); break;
-        case 1: collide_pop<T, 1>(c, hs, gs, ho, go); break;
-        case 2: collide_pop<T, 2>(c, hs, gs, ho, go); break;
-        case 3: collide_pop<T, 3>(c, hs, gs, ho, go); break;
-        case 4: collide_pop<T, 4>(c, hs, gs, ho, go); break;
-        case 5: collide_pop<T, 5>(c, hs, gs, ho, go); break;
-        case 6: collide_pop<T, 6>(c, hs, gs, ho, go); break;
-        case 7: collide_pop<T, 7>(c, hs, gs, ho, go); break;
-        default: collide_pop<T, 8>(c, hs, gs, ho, go); break;
-    }
+__device__ __forceinline__ void collide_rest(const CollidePrep<T> &c, T hs, T gs, V2<T> ds, T &ho, T &go) {
+    constexpr T wa = kW<T>(0), w3 = kW3<T>(0);
+    const T h = hs + fma(c.nomw, fma(c.nr, wa, hs), w3 * fma(c.nhuu, c.hA, c.hZ));
+    ho = h - ((ds.x + ds.y) + (h - hs));
+    go = gs + fma(c.nomw, fma(c.np, w3, gs), w3 * fma(c.nhuu, c.gA, c.gZ));
 }
 
 // Zeroth and first moments of the streamed g.  The first moments are summed
@@ -416,33 +433,33 @@ __device__ __forceinline__ void collide_pop_rt(const CollidePrep<T> &c, int a, T
 // floating point when the two are close (they share the pressure part
 // w_a 3p), so only the small momentum-carrying parts are rounded.
 template <typename T>
-__device__ __forceinline__ void g_moments(T g0, T g1, T g2, T g3, T g4, T g5, T g6, T g7, T g8,
-                                          T &sg, T &mx, T &my) {
-    const T d13 = g1 - g3, d24 = g2 - g4, d57 = g5 - g7, d68 = g6 - g8;
-    mx = d13 + (d57 - d68);  // e_x: +1, 3: -1, 5: +1, 6: -1, 7: -1, 8: +1
-    my = d24 + (d57 + d68);  // e_y: +2, 4: -1, 5: +1, 6: +1, 7: -1, 8: -1
-    sg = ((g0 + (g1 + g3)) + (g2 + g4)) + ((g5 + g7) + (g6 + g8));
+__device__ __forceinline__ void g_moments(T g0, const V2<T> *g, T &sg, T &mx, T &my) {
+    // pairs (1,3), (2,4), (5,7), (6,8): e_1 = (1,0), e_2 = (0,1), e_5 = (1,1), e_6 = (-1,1)
+    const T d13 = g[0].x - g[0].y, d24 = g[1].x - g[1].y, d57 = g[2].x - g[2].y, d68 = g[3].x - g[3].y;
+    mx = d13 + (d57 - d68);
+    my = d24 + (d57 + d68);
+    sg = ((g0 + (g[0].x + g[0].y)) + (g[1].x + g[1].y)) + ((g[2].x + g[2].y) + (g[3].x + g[3].y));
 }
 
+// Collision of a node whose streamed pairs are in registers, and its write:
+// the pairs to ho / go + q np and the rest populations to h0o / g0o.
 template <typename T>
-__device__ __forceinline__ void collide_node(const Phys<T> &P, const T *hs, const T *gs, T r,
-                                             T drx, T dry, T dmx, T dmy, T kx, T ky, T *hout,
-                                             T *gout, T &ux, T &uy, T &p) {
-    T sg, mx, my;
-    g_moments<T>(gs[0], gs[1], gs[2], gs[3], gs[4], gs[5], gs[6], gs[7], gs[8], sg, mx, my);
-    const CollidePrep<T> c = collide_prep<T>(P, sg, mx, my, r, drx, dry, dmx, dmy, kx, ky);
-    T dsum = T(0);  // sum of the h increments: zero in exact arithmetic
-#pragma unroll
-    for (int a = 1; a < 9; ++a) {
-        collide_pop_rt<T>(c, a, hs[a], gs[a], hout[a], gout[a]);
-        dsum += hout[a] - hs[a];
-    }
-    collide_pop_rt<T>(c, 0, hs[0], gs[0], hout[0], gout[0]);
-    dsum += hout[0] - hs[0];
-    hout[0] -= dsum;  // local mass: sum_a hbar_a = sum_a h*_a up to one rounding
-    ux = c.ux;
-    uy = c.uy;
-    p = c.p;
+__device__ __forceinline__ void collide_store(const CollidePrep<T> &c, const V2<T> *hs, const V2<T> *gs, T h0, T g0,
+                                              size_t np, V2<T> *ho, V2<T> *go, T *h0o, T *g0o) {
+    V2<T> ds = vset(T(0), T(0)), h, g;
+    collide_pair<T, 0>(c, hs[0], gs[0], h, g, ds);
+    ho[0] = h;
+    go[0] = g;
+    collide_pair<T, 1>(c, hs[1], gs[1], h, g, ds);
+    ho[np] = h;
+    go[np] = g;
+    collide_pair<T, 2>(c, hs[2], gs[2], h, g, ds);
+    ho[2 * np] = h;
+    go[2 * np] = g;
+    collide_pair<T, 3>(c, hs[3], gs[3], h, g, ds);
+    ho[3 * np] = h;
+    go[3 * np] = g;
+    collide_rest<T>(c, h0, g0, ds, *h0o, *g0o);
 }
 
 template <typename T, typename Topo>
@@ -459,34 +476,25 @@ struct CollideArgs {
 // Collision and write of one node of a general mesh from its streamed,
 // bounced-back g and the h* of k_rho.
 template <typename T, typename Topo>
-__device__ __forceinline__ void collide_write(const CollideArgs<T, Topo> &A, int32_t i, size_t np, const T *gs, T r,
-                                              T drx, T dry, T dmx, T dmy, T kx, T ky) {
+__device__ __forceinline__ void collide_write(const CollideArgs<T, Topo> &A, int32_t i, size_t np, T g0,
+                                              const V2<T> *gs, T r, T drx, T dry, T dmx, T dmy, T kx, T ky) {
     const size_t n = (size_t)A.m.n, si = A.m.slot(i);
-    T hs[9];
-    {
-        V2<T> hp[4];
-        const V2<T> *hsb = reinterpret_cast<const V2<T> *>(A.F.hs + np);
+    V2<T> hs[4];
+    const V2<T> *hsb = reinterpret_cast<const V2<T> *>(A.F.hs + np);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) hp[q] = hsb[q * np + si];
-        unpack_pairs<T>(A.F.hs[si], hp, hs);
-    }
-    T hout[9], gout[9], ux, uy, p;
-    collide_node<T>(A.P, hs, gs, r, drx, dry, dmx, dmy, kx, ky, hout, gout, ux, uy, p);
-    V2<T> *hb = reinterpret_cast<V2<T> *>(A.fout + np);
-    V2<T> *gb = reinterpret_cast<V2<T> *>(A.fout + 10 * np);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        hb[q * np + si] = vset(hout[pair_dir(q, 0)], hout[pair_dir(q, 1)]);
-        gb[q * np + si] = vset(gout[pair_dir(q, 0)], gout[pair_dir(q, 1)]);
-    }
-    A.fout[si] = hout[0];
-    A.fout[9 * np + si] = gout[0];
-    if (!(finite_val(r) && finite_val(ux) && finite_val(uy) && finite_val(p))) atomicOr(A.flag, 1);
+    for (int q = 0; q < 4; ++q) hs[q] = hsb[q * np + si];
+    const T h0 = A.F.hs[si];
+    T sg, mx, my;
+    g_moments<T>(g0, gs, sg, mx, my);
+    const CollidePrep<T> c = collide_prep<T>(A.P, sg, mx, my, r, drx, dry, dmx, dmy, kx, ky);
+    collide_store<T>(c, hs, gs, h0, g0, np, reinterpret_cast<V2<T> *>(A.fout + np) + si,
+                     reinterpret_cast<V2<T> *>(A.fout + 10 * np) + si, A.fout + si, A.fout + 9 * np + si);
+    if (!(finite_val(r) && finite_val(c.ux) && finite_val(c.uy) && finite_val(c.p))) atomicOr(A.flag, 1);
     if (A.mom) {
         A.mom[i] = r;
-        A.mom[n + i] = ux;
-        A.mom[2 * n + i] = uy;
-        A.mom[3 * n + i] = p;
+        A.mom[n + i] = c.ux;
+        A.mom[2 * n + i] = c.uy;
+        A.mom[3 * n + i] = c.p;
     }
 }
 
@@ -500,17 +508,15 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 2) k_collide(const _
     const int k = m.tag_of(i);
     pdl_wait();
     pdl_trigger();
-    T dmx, dmy, gs[9];
-    {
-        // g streamed here (the h code on the g half of the state); h* was
-        // streamed and bounced back by k_rho
-        V2<T> gp[4];
-        stream_pairs<T>(m, A.fin + 9 * np, np, i, A.P.dt, gp, [&](auto &&fn) { m.each(row, fn); });
-        unpack_pairs<T>(A.fin[9 * np + m.slot(i)], gp, gs);
-        if (k) bounce_back<T>(k, gs);
-    }
+    // g streamed here (the h code on the g half of the state); h* was
+    // streamed and bounced back by k_rho
+    T dmx, dmy;
+    V2<T> gs[4];
+    stream_pairs<T>(m, A.fin + 9 * np, np, i, A.P.dt, gs, [&](auto &&fn) { m.each(row, fn); });
+    const T g0 = A.fin[9 * np + m.slot(i)];
+    if (k) bounce_pairs<T>(k, gs);
     recover(m, row, A.F.mu, i, dmx, dmy);
-    collide_write<T>(A, i, np, gs, A.F.rho[i], A.F.drx[i], A.F.dry[i], dmx, dmy, A.F.kx[i], A.F.ky[i]);
+    collide_write<T>(A, i, np, g0, gs, A.F.rho[i], A.F.drx[i], A.F.dry[i], dmx, dmy, A.F.kx[i], A.F.ky[i]);
 }
 
 // Initial state: post-collision distributions are the equilibria of

@@ -401,96 +401,110 @@ __global__ void __launch_bounds__(256) k_mu3(const __grid_constant__ Topo m, Fie
 // Per-node scalars of the collision (3-D form of CollidePrep).
 template <typename T>
 struct Prep3 {
-    T r, u[3], p, omw, opw, hdt, X[3], dr[3], K[3], du[3], uX, uD, uK, uu, udu;
+    T r, u[3], p;
+    T nr, np, nomw, nhuu;
+    T X[3], hA, hZ, V[3], gA, B[3], gZ, G[3], du[3];
 };
+
+// The scalars for given moments and relaxation factors omw = 1 - w, opw = 1 + w.
+template <typename T>
+__device__ __forceinline__ void prep3_terms(const Phys3<T> &P, Prep3<T> &c, T omw, T opw, const T *dr, const T *dm,
+                                            const T *K) {
+    constexpr T cs2 = T(1) / T(3);
+    const T r = c.r, f = opw * (T(0.5) * P.dt), m = omw * r, hr = T(0.5) * opw * r;
+    T uX = T(0), uV = T(0), uK = T(0), uu = T(0), uG = T(0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        c.X[k] = f * (cs2 * dr[k] - r * dm[k]);
+        const T Kk = f * K[k];
+        c.V[k] = fma(T(3), Kk, f * dr[k]);
+        c.du[k] = P.g[k] * P.dt;
+        c.G[k] = hr * c.du[k];
+        c.B[k] = Kk + c.G[k];
+        uX += c.u[k] * c.X[k];
+        uV += c.u[k] * c.V[k];
+        uK += c.u[k] * Kk;
+        uu += c.u[k] * c.u[k];
+        uG += c.G[k] * (c.u[k] + T(0.5) * c.du[k]);
+    }
+    c.nr = -r;
+    c.np = -c.p;
+    c.nomw = -omw;
+    c.nhuu = T(-0.5) * uu;
+    c.hZ = -uX;
+    c.hA = fma(T(-3), uX, m);
+    c.gA = m - uV;
+    c.gZ = -uK - uG;
+}
 
 template <typename T>
 __device__ __forceinline__ Prep3<T> prep3(const Phys3<T> &P, T sg, const T *mg, T r, const T *dr,
                                           const T *dm, const T *K) {
-    constexpr T cs2 = T(1) / T(3);
     Prep3<T> c;
-    c.hdt = T(0.5) * P.dt;
+    const T hdt = T(0.5) * P.dt;
     c.r = r;
     const T inv_r = recip_rn(r);
     T ud = T(0);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        c.u[k] = (mg[k] + c.hdt * K[k] + c.hdt * r * P.g[k]) * inv_r;
+        c.u[k] = (mg[k] + hdt * K[k] + hdt * r * P.g[k]) * inv_r;
         ud += c.u[k] * dr[k];
     }
-    c.p = div3(sg + c.hdt * ud);  // correctly rounded: a rounded 1/3 is a gain on p (see kW3)
+    c.p = div3(sg + hdt * ud);  // correctly rounded: a rounded 1/3 is a gain on p (see kW3)
     T C = (r - P.rho_v) * P.inv_drho;
     C = C < T(0) ? T(0) : (C > T(1) ? T(1) : C);
     const T s = C * P.inv_tau_l + (T(1) - C) * P.inv_tau_v;  // 1/tau
     const T d = recip_rn(T(2) + s);
-    c.omw = T(2) * s * d;  // 1 - w
-    c.opw = T(4) * d;      // 1 + w
-    c.uX = c.uD = c.uK = c.uu = c.udu = T(0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        c.X[k] = cs2 * dr[k] - r * dm[k];
-        c.dr[k] = dr[k];
-        c.K[k] = K[k];
-        c.du[k] = P.g[k] * P.dt;
-        c.uX += c.u[k] * c.X[k];
-        c.uD += c.u[k] * dr[k];
-        c.uK += c.u[k] * K[k];
-        c.uu += c.u[k] * c.u[k];
-        c.udu += c.du[k] * (T(2) * c.u[k] + c.du[k]);
-    }
+    prep3_terms<T>(P, c, T(2) * s * d, T(4) * d, dr, dm, K);
     return c;
 }
 
-// Update of population a (same increment form as collide_pop).
+// e.v for pair q's first direction, by sums and differences of components
 template <typename T>
-__device__ __forceinline__ void collide_pop3(const Prep3<T> &c, int a, T hs, T gs, T &hout, T &gout) {
-    const T ex = T(e3x(a)), ey = T(e3y(a)), ez = T(e3z(a));
-    const T wa = w3<T>(a), w3a = w3x3<T>(a);
-    const T eu = ex * c.u[0] + ey * c.u[1] + ez * c.u[2];
-    const T gmw = w3a * (eu + T(1.5) * eu * eu - T(0.5) * c.uu);  // Gamma - w
-    const T gam3 = w3a + T(3) * gmw;                             // 3 Gamma
-    const T eX = ex * c.X[0] + ey * c.X[1] + ez * c.X[2];
-    const T eD = ex * c.dr[0] + ey * c.dr[1] + ez * c.dr[2];
-    const T eK = ex * c.K[0] + ey * c.K[1] + ez * c.K[2];
-    const T edu = ex * c.du[0] + ey * c.du[1] + ez * c.du[2];
-    const T Fa = c.hdt * (eX - c.uX) * gam3;
-    const T Ga = c.hdt * (eD - c.uD) * gmw + c.hdt * (eK - c.uK) * gam3;
-    const T Ba = T(0.5) * c.r * w3a * (edu + T(1.5) * edu * (T(2) * eu + edu) - T(0.5) * c.udu);
-    const T dh = fma(c.r, wa, -hs) + c.r * gmw;
-    const T dg = fma(w3a, c.p, -gs) + c.r * gmw;
-    hout = hs + (c.omw * dh + c.opw * Fa);
-    gout = gs + (c.omw * dg + c.opw * (Ga + Ba));
+__device__ __forceinline__ T dir_dot3(int q, const T *v) {
+    const int a = 2 * q + 1;
+    T s = T(0);
+    bool any = false;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int e = k == 0 ? e3x(a) : (k == 1 ? e3y(a) : e3z(a));
+        if (e != 0) {
+            const T t = e > 0 ? v[k] : -v[k];
+            s = any ? s + t : t;
+            any = true;
+        }
+    }
+    return s;
 }
 
-// Collision of the opposite pair q = (a, a+1), a = 2q+1, in packed
-// two-wide arithmetic: e_(a+1) = -e_a and equal weights, so the odd parts
-// (e.u, e.X, e.grad rho, e.K, e.du) flip sign between the lanes and the even
-// parts are shared (collide_pop3 on both members).
+// Collision of the opposite pair q = (a, a+1), a = 2q+1 (collide_pair's
+// arithmetic in three dimensions).
 template <typename T>
-__device__ __forceinline__ void collide_pair3(const Prep3<T> &c, int q, V2<T> hs, V2<T> gs, V2<T> &ho,
-                                              V2<T> &go) {
+__device__ __forceinline__ void collide_pair3(const Prep3<T> &c, int q, V2<T> hs, V2<T> gs, V2<T> &ho, V2<T> &go,
+                                              V2<T> &ds) {
     const int a = 2 * q + 1;
-    const T ex = T(e3x(a)), ey = T(e3y(a)), ez = T(e3z(a));
     const T wa = w3<T>(a), w3a = w3x3<T>(a);
-    const T eu = ex * c.u[0] + ey * c.u[1] + ez * c.u[2];
-    const T eX = ex * c.X[0] + ey * c.X[1] + ez * c.X[2];
-    const T eD = ex * c.dr[0] + ey * c.dr[1] + ez * c.dr[2];
-    const T eK = ex * c.K[0] + ey * c.K[1] + ez * c.K[2];
-    const T edu = ex * c.du[0] + ey * c.du[1] + ez * c.du[2];
-    const T even = T(1.5) * eu * eu - T(0.5) * c.uu;
-    const V2<T> gmw = vfma(vset(w3a, w3a), vset(eu, -eu), vset(w3a * even, w3a * even));  // Gamma - w
-    const V2<T> gam3 = vfma(vset(T(3), T(3)), gmw, vset(w3a, w3a));                       // 3 Gamma
-    const V2<T> Fa = vmul(vset(c.hdt * (eX - c.uX), c.hdt * (-eX - c.uX)), gam3);
-    const V2<T> Ga = vfma(vset(c.hdt * (eD - c.uD), c.hdt * (-eD - c.uD)), gmw,
-                          vmul(vset(c.hdt * (eK - c.uK), c.hdt * (-eK - c.uK)), gam3));
-    const T bev = T(1.5) * edu * (T(2) * eu + edu) - T(0.5) * c.udu;
-    const T hrw = T(0.5) * c.r * w3a;
-    const V2<T> Sg = vfma(vset(hrw, hrw), vset(edu + bev, bev - edu), Ga);  // G + B
-    const V2<T> rg = vmul(vset(c.r, c.r), gmw);
-    const V2<T> dh = vadd(vfma(vset(c.r, c.r), vset(wa, wa), vset(-hs.x, -hs.y)), rg);   // h_eq - h*
-    const V2<T> dg = vadd(vfma(vset(w3a, w3a), vset(c.p, c.p), vset(-gs.x, -gs.y)), rg);  // g_eq - g*
-    ho = vadd(hs, vfma(vset(c.omw, c.omw), dh, vmul(vset(c.opw, c.opw), Fa)));
-    go = vadd(gs, vfma(vset(c.omw, c.omw), dg, vmul(vset(c.opw, c.opw), Sg)));
+    const T eu = dir_dot3<T>(q, c.u), eX = dir_dot3<T>(q, c.X), eV = dir_dot3<T>(q, c.V), eB = dir_dot3<T>(q, c.B);
+    const T eG = dir_dot3<T>(q, c.G), ed = dir_dot3<T>(q, c.du);
+    const T qe = fma(T(1.5) * eu, eu, c.nhuu), eA = T(3) * eX;
+    const T ge = fma(eG, fma(T(1.5), ed, T(3) * eu), c.gZ);
+    const V2<T> qv = vset(qe + eu, qe - eu);
+    const V2<T> hz = vfma(qv, vset(c.hA + eA, c.hA - eA), vset(c.hZ + eX, c.hZ - eX));
+    const V2<T> gz = vfma(qv, vset(c.gA + eV, c.gA - eV), vset(ge + eB, ge - eB));
+    const V2<T> w32 = vset(w3a, w3a), nomw = vset(c.nomw, c.nomw);
+    ho = vadd(hs, vfma(nomw, vfma(vset(c.nr, c.nr), vset(wa, wa), hs), vmul(w32, hz)));
+    go = vadd(gs, vfma(nomw, vfma(vset(c.np, c.np), w32, gs), vmul(w32, gz)));
+    ds = vadd(ds, vfma(hs, vset(T(-1), T(-1)), ho));
+}
+
+// The rest population; its h takes the sum of the node's h increments (see
+// collide_rest).
+template <typename T>
+__device__ __forceinline__ void collide_rest3(const Prep3<T> &c, T hs, T gs, V2<T> ds, T &ho, T &go) {
+    const T wa = w3<T>(0), w3a = w3x3<T>(0);
+    const T h = hs + fma(c.nomw, fma(c.nr, wa, hs), w3a * fma(c.nhuu, c.hA, c.hZ));
+    ho = h - ((ds.x + ds.y) + (h - hs));
+    go = gs + fma(c.nomw, fma(c.np, w3a, gs), w3a * fma(c.nhuu, c.gA, c.gZ));
 }
 
 template <typename T, typename Topo>
@@ -549,20 +563,15 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 1) k_collide3(const 
     const Prep3<T> c = prep3<T>(A.P, sg, mg, r, dr, dm, K);
     V2<T> *hb = reinterpret_cast<V2<T> *>(A.fout + np);
     V2<T> *gb = reinterpret_cast<V2<T> *>(A.fout + 20 * np);
-    T dsum = T(0);
+    V2<T> ds = vset(T(0), T(0));
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         V2<T> ho, go;
-        collide_pair3<T>(c, q, hp[q], gp[q], ho, go);
-        dsum += (ho.x - hp[q].x) + (ho.y - hp[q].y);
+        collide_pair3<T>(c, q, hp[q], gp[q], ho, go, ds);
         hb[q * np + i] = ho;
         gb[q * np + i] = go;
     }
-    T hout0, gout0;
-    collide_pop3<T>(c, 0, h0, g0, hout0, gout0);
-    dsum += hout0 - h0;
-    A.fout[i] = hout0 - dsum;  // local mass: sum_a hbar_a = sum_a h*_a up to one rounding
-    A.fout[19 * np + i] = gout0;
+    collide_rest3<T>(c, h0, g0, ds, A.fout[i], A.fout[19 * np + i]);
     if (!(finite_val(r) && finite_val(c.u[0]) && finite_val(c.u[1]) && finite_val(c.u[2]) &&
           finite_val(c.p)))
         atomicOr(A.flag, 1);
@@ -589,40 +598,26 @@ __global__ void __launch_bounds__(128) k_init3(const __grid_constant__ Topo m, T
     for (int c = 0; c < 3; ++c) K[c] = F.k[c][i];
     const T r = mom[i];
     Prep3<T> c;
-    constexpr T cs2 = T(1) / T(3);
-    c.hdt = T(0.5) * P.dt;
     c.r = r;
     c.p = mom[4 * n + i];
-    c.uX = c.uD = c.uK = c.uu = c.udu = T(0);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        c.u[k] = mom[(1 + k) * n + i];
-        c.X[k] = cs2 * dr[k] - r * dm[k];
-        c.dr[k] = dr[k];
-        c.K[k] = K[k];
-        c.du[k] = P.g[k] * P.dt;
-        c.uX += c.u[k] * c.X[k];
-        c.uD += c.u[k] * dr[k];
-        c.uK += c.u[k] * K[k];
-        c.uu += c.u[k] * c.u[k];
-        c.udu += c.du[k] * (T(2) * c.u[k] + c.du[k]);
-    }
-    // eq + S: the collision increment form with 1 - w = 1 and 1 + w = 1
-    // applied to psi* = 0 gives eq + F (h) and eq + G + B (g)
-    c.omw = T(1);
-    c.opw = T(1);
-    T h[19], g[19];
-#pragma unroll
-    for (int a = 0; a < 19; ++a) collide_pop3<T>(c, a, T(0), T(0), h[a], g[a]);
+    for (int k = 0; k < 3; ++k) c.u[k] = mom[(1 + k) * n + i];
+    // eq + S: the collision's increment with 1 - w = 1 and 1 + w = 1 from
+    // psi* = 0
+    prep3_terms<T>(P, c, T(1), T(1), dr, dm, K);
     V2<T> *hb = reinterpret_cast<V2<T> *>(fout + np);
     V2<T> *gb = reinterpret_cast<V2<T> *>(fout + 20 * np);
+    const V2<T> zero = vset(T(0), T(0));
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-        hb[q * np + i] = vset(h[2 * q + 1], h[2 * q + 2]);
-        gb[q * np + i] = vset(g[2 * q + 1], g[2 * q + 2]);
+        V2<T> h, g, ds = zero;
+        collide_pair3<T>(c, q, zero, zero, h, g, ds);
+        hb[q * np + i] = h;
+        gb[q * np + i] = g;
     }
-    fout[i] = h[0];
-    fout[19 * np + i] = g[0];
+    const T wa = w3<T>(0), w3a = w3x3<T>(0);
+    fout[i] = fma(r, wa, w3a * fma(c.nhuu, c.hA, c.hZ));
+    fout[19 * np + i] = fma(c.p, w3a, w3a * fma(c.nhuu, c.gA, c.gZ));
 }
 
 // Moments in caller order, FP64: out[0..N) rho, [N..2N) C, [2N..5N) u

@@ -49,6 +49,15 @@ struct LatCoef {
     T r[3][6][2];      // recovery coefficients
 };
 
+// Weights of the uniform split's streaming (stream_uni_v), per direction of
+// a pair: ka = (-dt/(6h), dt/(6h)) (odd part), kb = dt^2/(2h^2) (even part).
+template <typename T>
+struct StreamUni {
+    V2<T> ka, nkb;     // ka, -kb
+    V2<T> a2p, a2m;    // kb + 2 ka, kb - 2 ka
+    V2<T> a3p, a3m;    // 2 kb + 3 ka, 2 kb - 3 ka
+};
+
 template <typename T>
 struct LatArgs {
     int32_t nx, ny, walls;
@@ -71,8 +80,7 @@ struct LatArgs {
     // tiles when uni is set (the host checked the mesh's interior weights)
     int32_t uni;
     T al;        // 1 / (6 h)
-    V2<T> ka;    // (-dt/(6h), dt/(6h)): odd part of the streaming weights
-    V2<T> kb;    // (dt^2/(2h^2), dt^2/(2h^2)): even part
+    StreamUni<T> su;
     // FP64 kappa lap rho term of mu (FELBM_PARAM_LAP_FP64; read only by the
     // kernel built for it): 1/(6h), kappa and the recovery coefficients
     double al64, kappa64;
@@ -96,8 +104,14 @@ struct LatArgs {
 //   (e.(h^2 b_o).e) d_o:  q0 e = (1,0): SA = 2E_0 + E_1 - E_2, SB = S_0;
 //   q1 (0,1): -E_0 + E_1 + 2E_2, S_2;  q2 (1,1): E_0 + 2E_1 + E_2, S_1;
 //   q3 (-1,1): 3(E_2 - E_0), 2(S_0 + S_2) - S_1.
+// Terms of one neighbour are collected where that saves operations (d_o =
+// f(o) - f, E_k = d_k - d_{k+3}):
+//   q0: (kb + 2ka) d_0 + (kb - 2ka) d_3 + ka (E_1 - E_2), and q1, q2 alike;
+//   q3: (2kb + 3ka)(d_2 + d_3) + (2kb - 3ka)(d_0 + d_5) - kb (d_1 + d_4)
+// (40 packed operations for the four pairs against 47 with the sums SA, SB).
 // Only differences of neighbouring values are rounded, as in the weighted
-// difference form of the tables (exact for constant fields); no weight is
+// difference form of the tables (exact for constant fields), and the sum of
+// the weighted differences is added to psi in one rounding; no weight is
 // loaded.  Opposite offsets carry opposite recovery weights, so a recovered
 // derivative needs three differences instead of six.
 
@@ -110,41 +124,31 @@ __device__ __forceinline__ V2<T> vsub(V2<T> a, V2<T> b) {
 // the offsets o = (1,0), (1,1), (0,1), (-1,0), (-1,-1), (0,-1)
 template <typename T, int Q>
 __device__ __forceinline__ V2<T> stream_uni_v(V2<T> s, V2<T> n0, V2<T> n1, V2<T> n2, V2<T> n3, V2<T> n4,
-                                              V2<T> n5, V2<T> ka, V2<T> kb) {
-    const V2<T> two = vset(T(2), T(2));
-    if (Q == 0) {
-        const V2<T> SA = vfma(vsub<T>(n0, n3), two, vsub<T>(vsub<T>(n1, n4), vsub<T>(n2, n5)));
-        const V2<T> SB = vadd(vsub<T>(n0, s), vsub<T>(n3, s));
-        return vfma(ka, SA, vfma(kb, SB, s));
-    } else if (Q == 1) {
-        const V2<T> SA = vfma(vsub<T>(n2, n5), two, vsub<T>(vsub<T>(n1, n4), vsub<T>(n0, n3)));
-        const V2<T> SB = vadd(vsub<T>(n2, s), vsub<T>(n5, s));
-        return vfma(ka, SA, vfma(kb, SB, s));
-    } else if (Q == 2) {
-        const V2<T> SA = vfma(vsub<T>(n1, n4), two, vadd(vsub<T>(n0, n3), vsub<T>(n2, n5)));
-        const V2<T> SB = vadd(vsub<T>(n1, s), vsub<T>(n4, s));
-        return vfma(ka, SA, vfma(kb, SB, s));
-    } else {
-        const V2<T> d0 = vsub<T>(n0, s), d1 = vsub<T>(n1, s), d2 = vsub<T>(n2, s);
-        const V2<T> d3 = vsub<T>(n3, s), d4 = vsub<T>(n4, s), d5 = vsub<T>(n5, s);
-        const V2<T> S02 = vadd(vadd(d0, d3), vadd(d2, d5));
-        const V2<T> SB = vsub<T>(vadd(S02, S02), vadd(d1, d4));
-        const V2<T> SA = vsub<T>(vadd(d2, d3), vadd(d0, d5));  // E_2 - E_0
-        return vfma(vmul(ka, vset(T(3), T(3))), SA, vfma(kb, SB, s));
+                                              V2<T> n5, const StreamUni<T> &u) {
+    if (Q == 3) {
+        const V2<T> a = vadd(vsub<T>(n2, s), vsub<T>(n3, s)), b = vadd(vsub<T>(n0, s), vsub<T>(n5, s));
+        const V2<T> c = vadd(vsub<T>(n1, s), vsub<T>(n4, s));
+        return vadd(s, vfma(u.a3p, a, vfma(u.a3m, b, vmul(u.nkb, c))));
     }
+    // the pair's own axis (np, nm), and the odd part of the other two offsets
+    const V2<T> np = Q == 0 ? n0 : (Q == 1 ? n2 : n1), nm = Q == 0 ? n3 : (Q == 1 ? n5 : n4);
+    const V2<T> odd = Q == 0   ? vsub<T>(vsub<T>(n1, n4), vsub<T>(n2, n5))
+                      : Q == 1 ? vsub<T>(vsub<T>(n1, n4), vsub<T>(n0, n3))
+                               : vadd(vsub<T>(n0, n3), vsub<T>(n2, n5));
+    return vadd(s, vfma(u.a2p, vsub<T>(np, s), vfma(u.a2m, vsub<T>(nm, s), vmul(u.ka, odd))));
 }
 
 // streamed pair Q of the node at index c of a window with rows of W pairs
 template <typename T, int W, int Q>
-__device__ __forceinline__ V2<T> stream_uni(const V2<T> *b, int c, V2<T> ka, V2<T> kb) {
-    return stream_uni_v<T, Q>(b[c], b[c + 1], b[c + W + 1], b[c + W], b[c - 1], b[c - W - 1], b[c - W], ka, kb);
+__device__ __forceinline__ V2<T> stream_uni(const V2<T> *b, int c, const StreamUni<T> &u) {
+    return stream_uni_v<T, Q>(b[c], b[c + 1], b[c + W + 1], b[c + W], b[c - 1], b[c - W - 1], b[c - W], u);
 }
 
 // The same for three nodes stacked in one column, from 13 loads instead of
 // 21: rb[j] is the offset of the window row holding y - 1 + j (j = 0 .. 4,
 // y the first node's row), c the column.
 template <typename T, int Q>
-__device__ __forceinline__ void stream_uni3(const V2<T> *b, const int *rb, int c, V2<T> ka, V2<T> kb, V2<T> *out) {
+__device__ __forceinline__ void stream_uni3(const V2<T> *b, const int *rb, int c, const StreamUni<T> &u, V2<T> *out) {
     V2<T> cx[5], cl[4], cr[4];
 #pragma unroll
     for (int j = 0; j < 5; ++j) cx[j] = b[rb[j] + c];
@@ -155,7 +159,7 @@ __device__ __forceinline__ void stream_uni3(const V2<T> *b, const int *rb, int c
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-        out[i] = stream_uni_v<T, Q>(cx[i + 1], cr[i], cr[i + 1], cx[i + 2], cl[i + 1], cl[i], cx[i], ka, kb);
+        out[i] = stream_uni_v<T, Q>(cx[i + 1], cr[i], cr[i + 1], cx[i + 2], cl[i + 1], cl[i], cx[i], u);
 }
 
 // (6h R_x f, 6h R_y f) from the six neighbour values
@@ -194,11 +198,18 @@ inline void lat_uniform_consts(const StructuredInfo &si, double dt, LatArgs<T> &
     const double h = si.h;
     A.uni = lattice_uniform(si) ? 1 : 0;
     A.al = (T)(1.0 / (6.0 * h));
-    const double ka = dt / (6.0 * h), kb = dt * dt / (2.0 * h * h);
-    A.ka.x = (T)-ka;
-    A.ka.y = (T)ka;
-    A.kb.x = (T)kb;
-    A.kb.y = (T)kb;
+    const double kb = dt * dt / (2.0 * h * h);
+    auto set = [](V2<T> &v, double x, double y) {
+        v.x = (T)x;
+        v.y = (T)y;
+    };
+    const double k = dt / (6.0 * h);
+    set(A.su.ka, -k, k);
+    set(A.su.nkb, -kb, -kb);
+    set(A.su.a2p, kb - 2.0 * k, kb + 2.0 * k);
+    set(A.su.a2m, kb + 2.0 * k, kb - 2.0 * k);
+    set(A.su.a3p, 2.0 * kb - 3.0 * k, 2.0 * kb + 3.0 * k);
+    set(A.su.a3m, 2.0 * kb + 3.0 * k, 2.0 * kb - 3.0 * k);
 }
 
 __device__ __forceinline__ int lat_kind(int walls, int y, int ny) {
@@ -428,40 +439,6 @@ __device__ __forceinline__ V2<T> stream_pair(const LatCoef<T> &cf, int k, int q,
     return vfma(vset(-dt, -dt), acc, self);
 }
 
-// Collision of the opposite pair q = (a, abar) of one node (see
-// collide_pop): e_abar = -e_a and w_abar = w_a, so the odd parts (e.u, e.X,
-// e.grad rho, e.K, e.du) flip sign between the two lanes and the even parts
-// are shared; the two lanes run in packed two-wide arithmetic.
-template <typename T, int Q>
-__device__ __forceinline__ void collide_pair(const CollidePrep<T> &c, V2<T> hs, V2<T> gs, V2<T> &ho,
-                                             V2<T> &go) {
-    constexpr int A = pair_dir(Q, 0);
-    constexpr int ex = kEx(A), ey = kEy(A);
-    constexpr T wa = kW<T>(A), w3 = kW3<T>(A);
-    const T eu = T(ex) * c.ux + T(ey) * c.uy;
-    const T eX = T(ex) * c.Xx + T(ey) * c.Xy;
-    const T eD = T(ex) * c.drx + T(ey) * c.dry;
-    const T eK = T(ex) * c.kx + T(ey) * c.ky;
-    const T edu = T(ex) * c.dux + T(ey) * c.duy;
-    // Gamma - w = 3w (e.u + 1.5 (e.u)^2 - 0.5 u.u), formed without the w
-    // offset (FP32: keeps the momentum part); 3w from kW3
-    const T even = T(1.5) * eu * eu - T(0.5) * c.uu;
-    const V2<T> gmw = vfma(vset(w3, w3), vset(eu, -eu), vset(w3 * even, w3 * even));
-    const V2<T> gam3 = vfma(vset(T(3), T(3)), gmw, vset(w3, w3));  // 3 Gamma
-    const V2<T> Fa = vmul(vset(c.hdt * (eX - c.uX), c.hdt * (-eX - c.uX)), gam3);
-    const V2<T> Ga = vfma(vset(c.hdt * (eD - c.uD), c.hdt * (-eD - c.uD)), gmw,
-                          vmul(vset(c.hdt * (eK - c.uK), c.hdt * (-eK - c.uK)), gam3));
-    // 1/2 [g_eq(u + du) - g_eq(u)] = rho/2 [Gamma(u + du) - Gamma(u)]
-    const T bev = T(1.5) * edu * (T(2) * eu + edu) - T(0.5) * c.udu;
-    const T hrw = T(0.5) * c.r * w3;
-    const V2<T> Sg = vfma(vset(hrw, hrw), vset(edu + bev, bev - edu), Ga);
-    const V2<T> rg = vmul(vset(c.r, c.r), gmw);
-    const V2<T> dh = vadd(vfma(vset(c.r, c.r), vset(wa, wa), vset(-hs.x, -hs.y)), rg);  // h_eq - h*
-    const V2<T> dg = vadd(vfma(vset(w3, w3), vset(c.p, c.p), vset(-gs.x, -gs.y)), rg);  // g_eq - g*
-    ho = vadd(hs, vfma(vset(c.omw, c.omw), dh, vmul(vset(c.opw, c.opw), Fa)));
-    go = vadd(gs, vfma(vset(c.omw, c.omw), dg, vmul(vset(c.opw, c.opw), Sg)));
-}
-
 // Bounce-back of a pair at a wall row of kind k (1: inward normal +y, the
 // slot-0 directions 2, 5, 6 of pairs 1..3 take their opposites; 2: normal
 // -y, the slot-1 directions 4, 7, 8 take theirs).
@@ -558,33 +535,26 @@ __device__ __forceinline__ void lat_node(const LatArgs<T> &A, const LatCoef<T> &
     const int c = (ly + 1) * PG::W + lx + PG::XH;
     V2<T> gq[4];
     if (UNI) {
-        gq[0] = stream_uni<T, PG::W, 0>(gT + 0 * PG::N, c, A.ka, A.kb);
-        gq[1] = stream_uni<T, PG::W, 1>(gT + 1 * PG::N, c, A.ka, A.kb);
-        gq[2] = stream_uni<T, PG::W, 2>(gT + 2 * PG::N, c, A.ka, A.kb);
-        gq[3] = stream_uni<T, PG::W, 3>(gT + 3 * PG::N, c, A.ka, A.kb);
+        gq[0] = stream_uni<T, PG::W, 0>(gT + 0 * PG::N, c, A.su);
+        gq[1] = stream_uni<T, PG::W, 1>(gT + 1 * PG::N, c, A.su);
+        gq[2] = stream_uni<T, PG::W, 2>(gT + 2 * PG::N, c, A.su);
+        gq[3] = stream_uni<T, PG::W, 3>(gT + 3 * PG::N, c, A.su);
     } else {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             gq[q] = bounce_pair<T>(k, q, stream_pair<T, PG::W>(C, k, q, gT + q * PG::N, c, P.dt));
     }
     T sg, mx, my;
-    // g_1 = q0.x, g_3 = q0.y, g_2 = q1.x, g_4 = q1.y, g_5 = q2.x, g_7 = q2.y, g_6 = q3.x, g_8 = q3.y
-    g_moments<T>(g0, gq[0].x, gq[1].x, gq[0].y, gq[1].y, gq[2].x, gq[3].x, gq[2].y, gq[3].y, sg, mx, my);
+    g_moments<T>(g0, gq, sg, mx, my);
     const CollidePrep<T> cp = collide_prep<T>(P, sg, mx, my, r0, drx, dry, dmx, dmy, kx, ky);
     const T r = cp.r, ux = cp.ux, uy = cp.uy, p = cp.p;
-    // pairs, then the rest population, which also takes the sum of the h
-    // increments (zero in exact arithmetic): the collision then keeps the
-    // node's mass to one rounding instead of accumulating the rounding of the
-    // nine source terms every step
-    T dsum = T(0);
+    V2<T> ds = vset(T(0), T(0));
     V2<T> *hout = reinterpret_cast<V2<T> *>(A.fout + np);
     V2<T> *gout = reinterpret_cast<V2<T> *>(A.fout + 10 * np);
     auto pair_update = [&](auto qc) {
         constexpr int q = decltype(qc)::value;
-        const V2<T> hs = s_psi[q][tid];
         V2<T> ho, go;
-        collide_pair<T, q>(cp, hs, gq[q], ho, go);
-        dsum += (ho.x - hs.x) + (ho.y - hs.y);
+        collide_pair<T, q>(cp, s_psi[q][tid], gq[q], ho, go, ds);
         hout[(size_t)q * np + ip] = ho;
         gout[(size_t)q * np + ip] = go;
     };
@@ -592,13 +562,7 @@ __device__ __forceinline__ void lat_node(const LatArgs<T> &A, const LatCoef<T> &
     pair_update(IntC<1>{});
     pair_update(IntC<2>{});
     pair_update(IntC<3>{});
-    {
-        T ho, go;
-        collide_pop_rt<T>(cp, 0, h0, g0, ho, go);
-        dsum += ho - h0;
-        A.fout[ip] = ho - dsum;
-        A.fout[9 * np + ip] = go;
-    }
+    collide_rest<T>(cp, h0, g0, ds, A.fout[ip], A.fout[9 * np + ip]);
     if (!(finite_val(r) && finite_val(ux) && finite_val(uy) && finite_val(p))) atomicOr(A.flag, 1);
     if (A.mom) {
         A.mom[i] = r;
@@ -752,7 +716,7 @@ __device__ __forceinline__ bool lat_tile_impl(const LatArgs<T> &A, const LatCoef
                 auto pair = [&](auto qc) {
                     constexpr int p = decltype(qc)::value;
                     V2<T> v[3];
-                    stream_uni3<T, p>(hT + p * PH::N, rb, c, A.ka, A.kb, v);
+                    stream_uni3<T, p>(hT + p * PH::N, rb, c, A.su, v);
 #pragma unroll
                     for (int i = 0; i < 3; ++i) {
                         const T t = v[i].x + v[i].y;

@@ -105,11 +105,10 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
     const size_t np = pad4(m.slots());
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
-    T gs[9];
+    V2<T> gs[4];
     {
         const int e0 = own ? sb[tid >> 5] + (tid & 31) : 0;
-        V2<T> gp[4];
-        stream_pairs<T>(m, A.c.fin + 9 * np, np, g, A.c.P.dt, gp, [&](auto &&fn) {
+        stream_pairs<T>(m, A.c.fin + 9 * np, np, g, A.c.P.dt, gs, [&](auto &&fn) {
             m.template each_get<false>(row, fn, [&](int k, Ell2<T>) {
                 Ell2<T> v{T(0), T(0)};
                 if (k < row.deg) {
@@ -119,9 +118,9 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
                 return v;
             });
         });
-        unpack_pairs<T>(A.c.fin[9 * np + g], gp, gs);
-        if (tag) bounce_back<T>(tag, gs);
+        if (tag) bounce_pairs<T>(tag, gs);
     }
+    const T g0 = A.c.fin[9 * np + g];
     if (tid < n3) rho[tid] = own ? rho_own : grho[__ldg(A.node + base + tid)];
     if (tid + kPatch < n3) rho[tid + kPatch] = rho1;
     for (int32_t r = tid + 2 * kPatch; r < n3; r += kPatch) {
@@ -180,7 +179,7 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
         each(tid, n1, [&](int j, V2<CT> a) { grad_edge<T>((T)a.x, (T)a.y, mu[j] - fi, dmx, dmy); });
     }
     const V2<T> gr = grd[tid];
-    collide_write<T>(A.c, g, np, gs, rho_own, gr.x, gr.y, dmx, dmy, kx_own, ky_own);
+    collide_write<T>(A.c, g, np, g0, gs, rho_own, gr.x, gr.y, dmx, dmy, kx_own, ky_own);
 }
 
 }  // namespace felbm
