@@ -10,6 +10,7 @@
 #include "felbm_internal.h"
 #include "felbm_kernels.cuh"
 #include "felbm_lattice.cuh"
+#include "felbm_latpass.cuh"
 #include "felbm_patch.cuh"
 
 using namespace felbm;
@@ -316,6 +317,30 @@ static void step_lattice(felbm_state *s, LatArgs<T> &A, bool write_mom) {
     s->cur ^= 1;
 }
 
+// One FP64 step of a lattice: its passes.  Few nodes are spread over the SMs
+// in small blocks.
+template <int S>
+static void launch_pass(felbm_state *s, const LatArgs<double> &A) {
+    int32_t lo, hi;
+    pass_rows(A.ny, A.gny, A.ylo, A.yhi, 3 - S, lo, hi);
+    const int64_t nodes = (int64_t)(hi - lo) * A.nx;
+    const int bs = nodes >= 152 * 512 ? kPassBlock : (nodes >= 152 * 128 ? 64 : 32);
+    const int sl = prof_begin(s, S);
+    launch_pdl(k_lat_pass<double, S>, nblocks(nodes, bs), bs, 0, s->mesh->stream, A);
+    prof_end(s, sl);
+}
+
+static void step_lattice64(felbm_state *s, LatArgs<double> &A, bool write_mom) {
+    A.fin = reinterpret_cast<const double *>(s->f[s->cur]);
+    A.fout = reinterpret_cast<double *>(s->f[s->cur ^ 1]);
+    A.mom = write_mom ? reinterpret_cast<double *>(s->mom) : nullptr;
+    launch_pass<0>(s, A);
+    launch_pass<1>(s, A);
+    launch_pass<2>(s, A);
+    launch_pass<3>(s, A);
+    s->cur ^= 1;
+}
+
 // The dynamic shared memory of k_lat_step is above the default limit: set
 // the function attribute once per device (bit d of done, set only once the
 // call succeeded; devices from 64 on set it at every call).  A refusal is
@@ -396,11 +421,8 @@ static int do_steps(felbm_state *s, int64_t n) {
     }
     if (m->kind == 1) {
         const bool l64 = lap_fp64(s);
-        cudaError_t ea;
-        if constexpr (sizeof(T) == 4)
-            ea = l64 ? lat_smem_attr<T, true>() : lat_smem_attr<T, false>();
-        else
-            ea = lat_smem_attr<T, false>();
+        cudaError_t ea = cudaSuccess;
+        if constexpr (sizeof(T) == 4) ea = l64 ? lat_smem_attr<T, true>() : lat_smem_attr<T, false>();
         if (ea != cudaSuccess) return cuda_status(ea);
         LatArgs<T> A;
         A.nx = m->sinfo.nx;
@@ -414,7 +436,7 @@ static int do_steps(felbm_state *s, int64_t n) {
         A.c = lat_coef<T>(m, s->params.dt);
         lat_uniform_consts<T>(m->sinfo, s->params.dt, A);
         A.P = phys_of<T>(s->params);
-        A.rho = fields_of<T>(s).rho;
+        A.rho = reinterpret_cast<T *>(s->scratch);
         A.flag = s->d_flag;
         A.al64 = 1.0 / (6.0 * m->sinfo.h);
         A.kappa64 = kappa64(s->params);
@@ -422,13 +444,12 @@ static int do_steps(felbm_state *s, int64_t n) {
             for (int o = 0; o < 6; ++o)
                 for (int c = 0; c < 2; ++c) A.r64[k][o][c] = m->sinfo.a[k][o][c];
         for (int64_t k = 0; k < n; ++k) {
-            if constexpr (sizeof(T) == 4) {
-                if (l64) {
-                    step_lattice<T, true>(s, A, k == n - 1);
-                    continue;
-                }
-            }
-            step_lattice<T, false>(s, A, k == n - 1);
+            if constexpr (sizeof(T) == 8)
+                step_lattice64(s, A, k == n - 1);
+            else if (l64)
+                step_lattice<T, true>(s, A, k == n - 1);
+            else
+                step_lattice<T, false>(s, A, k == n - 1);
         }
     } else {
         const DevELL<T> d = dev_ell<T>(m);

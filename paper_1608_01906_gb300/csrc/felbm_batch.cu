@@ -21,6 +21,7 @@
 #include "felbm_internal.h"
 #include "felbm_kernels.cuh"
 #include "felbm_lattice.cuh"
+#include "felbm_latpass.cuh"
 
 namespace felbm {
 
@@ -138,6 +139,18 @@ __global__ void __launch_bounds__(kNT, (sizeof(T) == 4 ? 1024 : 512) / kNT) k_ba
     lat_tile<T>(sA, batch_coef<T, SC>(B, sA), r.bx, r.by, S, bdsm, pp, none);
 }
 
+// A pass of an FP64 step over the whole batch: block b covers the kBatchPass
+// nodes from kBatchPass (bx + 65536 by) of its mesh (B.tiles).
+constexpr int kBatchPass = 64;
+template <int S>
+__global__ void __launch_bounds__(kBatchPass) k_batch_pass(const __grid_constant__ BatchArgs<double> B) {
+    __shared__ __align__(16) LatArgs<double> sA;
+    const TileRef r = B.tiles[blockIdx.x];
+    int cur = -1;
+    load_mesh<double>(B, r.mesh, sA, cur);
+    lat_pass<double, S>(sA, ((int64_t)r.bx + 65536 * (int64_t)r.by) * kBatchPass + threadIdx.x);
+}
+
 template <typename T>
 static LatCoef<T> lat_coef_b(const felbm_mesh *m, double dt) {
     LatCoef<T> c;
@@ -194,7 +207,7 @@ struct felbm_batch {
     unsigned *d_ctr = nullptr;  // tile counters of the launches, by parity
     int32_t ntiles = 0;
     int parity = 0;
-    int sm_count = 0, max_bps = 1;
+    int sm_count = 0, max_bps = 0;  // (FP64 batches: passes, one block per entry of the list)
     int bps = 1, order = 0;  // chosen configuration (bps 0: one block per tile)
     bool autotune = false, tuned = false;
     double tuned_ms = 0.0;
@@ -216,12 +229,8 @@ static int b_status(cudaError_t e) {
     return FELBM_ERR_CUDA;
 }
 
-static size_t batch_smem(int esize) {
-    return esize == 8 ? lat_smem<double>() : lat_smem<float>();
-}
-
 template <typename T>
-static cudaError_t batch_launch(felbm_batch *b, int parity, int write_mom) {
+static BatchArgs<T> batch_args(felbm_batch *b, int parity, int write_mom) {
     BatchArgs<T> B;
     B.meshes = reinterpret_cast<const BatchMesh<T> *>(b->d_meshes);
     B.tiles = b->d_tiles;
@@ -231,26 +240,40 @@ static cudaError_t batch_launch(felbm_batch *b, int parity, int write_mom) {
     B.write_mom = write_mom;
     std::memset(&B.c, 0, sizeof(B.c));
     if (b->shared_coef) std::memcpy(&B.c, b->coef.data(), sizeof(B.c));
+    return B;
+}
+
+static cudaError_t batch_launch32(felbm_batch *b, int parity, int write_mom) {
+    const BatchArgs<float> B = batch_args<float>(b, parity, write_mom);
     b->launches++;
     const dim3 blk(kLTX, kLTY);
-    const size_t sm = batch_smem(sizeof(T));
+    const size_t sm = lat_smem<float>();
     if (b->bps > 0) {
         const unsigned grid = (unsigned)(b->bps * b->sm_count);
         if (b->shared_coef)
-            k_batch_step<T, true><<<grid, blk, sm, b->stream>>>(B);
+            k_batch_step<float, true><<<grid, blk, sm, b->stream>>>(B);
         else
-            k_batch_step<T, false><<<grid, blk, sm, b->stream>>>(B);
+            k_batch_step<float, false><<<grid, blk, sm, b->stream>>>(B);
     } else if (b->shared_coef) {
-        k_batch_tile<T, true><<<(unsigned)b->ntiles, blk, sm, b->stream>>>(B);
+        k_batch_tile<float, true><<<(unsigned)b->ntiles, blk, sm, b->stream>>>(B);
     } else {
-        k_batch_tile<T, false><<<(unsigned)b->ntiles, blk, sm, b->stream>>>(B);
+        k_batch_tile<float, false><<<(unsigned)b->ntiles, blk, sm, b->stream>>>(B);
     }
     return cudaGetLastError();
 }
 
+static cudaError_t batch_launch64(felbm_batch *b, int parity, int write_mom) {
+    const BatchArgs<double> B = batch_args<double>(b, parity, write_mom);
+    b->launches += 4;
+    k_batch_pass<0><<<(unsigned)b->ntiles, kBatchPass, 0, b->stream>>>(B);
+    k_batch_pass<1><<<(unsigned)b->ntiles, kBatchPass, 0, b->stream>>>(B);
+    k_batch_pass<2><<<(unsigned)b->ntiles, kBatchPass, 0, b->stream>>>(B);
+    k_batch_pass<3><<<(unsigned)b->ntiles, kBatchPass, 0, b->stream>>>(B);
+    return cudaGetLastError();
+}
+
 static cudaError_t launch_any(felbm_batch *b, int parity, int write_mom) {
-    return b->esize == 8 ? batch_launch<double>(b, parity, write_mom)
-                         : batch_launch<float>(b, parity, write_mom);
+    return b->esize == 8 ? batch_launch64(b, parity, write_mom) : batch_launch32(b, parity, write_mom);
 }
 
 static cudaError_t upload_tiles(felbm_batch *b) {
@@ -325,20 +348,20 @@ static int setup_meshes(felbm_batch *b) {
     return b_status(cudaMemcpy(b->d_meshes, hm.data(), n * sizeof(BatchMesh<T>), cudaMemcpyHostToDevice));
 }
 
-template <typename T>
+// FP32: shared memory and the co-resident maximum of the walking kernel.
 static int occupancy(felbm_batch *b) {
     int bps = 0;
-    const int sm = (int)batch_smem(sizeof(T));
-    cudaError_t e = cudaFuncSetAttribute(k_batch_tile<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    const int sm = (int)lat_smem<float>();
+    cudaError_t e = cudaFuncSetAttribute(k_batch_tile<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_batch_tile<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        e = cudaFuncSetAttribute(k_batch_tile<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_batch_step<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        e = cudaFuncSetAttribute(k_batch_step<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_batch_step<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        e = cudaFuncSetAttribute(k_batch_step<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_batch_step<T, false>, kLTX * kLTY,
-                                                          batch_smem(sizeof(T)));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_batch_step<float, false>, kLTX * kLTY,
+                                                          (size_t)sm);
     if (e != cudaSuccess) return b_status(e);
     b->max_bps = std::max(1, bps);
     return FELBM_OK;
@@ -397,9 +420,14 @@ int felbm_batch_create(felbm_state *const *states, int32_t n_states, uint32_t fl
     for (int32_t k = 0; k < n_states; ++k) {
         const int tx = (states[k]->mesh->sinfo.nx + kLTX - 1) / kLTX;
         const int ty = (states[k]->mesh->sinfo.ny + kLTY - 1) / kLTY;
-        for (int by = 0; by < ty; ++by)
-            for (int bx = 0; bx < tx; ++bx)
-                per[k].push_back(TileRef{(uint16_t)k, (uint16_t)bx, (uint16_t)by, 0});
+        if (b->esize == 8) {  // blocks of the passes
+            for (int64_t q = 0; q * kBatchPass < states[k]->mesh->n_nodes; ++q)
+                per[k].push_back(TileRef{(uint16_t)k, (uint16_t)(q & 65535), (uint16_t)(q >> 16), 0});
+        } else {
+            for (int by = 0; by < ty; ++by)
+                for (int bx = 0; bx < tx; ++bx)
+                    per[k].push_back(TileRef{(uint16_t)k, (uint16_t)bx, (uint16_t)by, 0});
+        }
         b->tiles_mesh_major.insert(b->tiles_mesh_major.end(), per[k].begin(), per[k].end());
     }
     {
@@ -425,7 +453,7 @@ int felbm_batch_create(felbm_state *const *states, int32_t n_states, uint32_t fl
     if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_ctr, 2 * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(b->d_ctr, 0, 2 * sizeof(unsigned));
     int st = b_status(e);
-    if (st == FELBM_OK) st = b->esize == 8 ? occupancy<double>(b) : occupancy<float>(b);
+    if (st == FELBM_OK && b->esize == 4) st = occupancy(b);
     if (st == FELBM_OK) {
         b->bps = b->max_bps;
         b->order = 0;
@@ -521,7 +549,7 @@ int felbm_batch_step(felbm_batch *b, int64_t n_steps) {
         for (int64_t p = 0; p < pairs && e == cudaSuccess; ++p) {
             if (b->graph) {
                 e = cudaGraphLaunch(b->graph, b->stream);
-                b->launches += 2;
+                b->launches += b->esize == 8 ? 8 : 2;
             } else {
                 e = launch_any(b, 0, 0);
                 if (e == cudaSuccess) e = launch_any(b, 1, 0);

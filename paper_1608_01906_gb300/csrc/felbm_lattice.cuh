@@ -72,7 +72,7 @@ struct LatArgs {
     Phys<T> P;
     const T *fin;
     T *fout;
-    T *rho;  // unused by the lattice step (rho is formed per tile)
+    T *rho;  // scratch fields of the FP64 passes (felbm_latpass.cuh); unused by the tile step
     T *mom;  // 4N or nullptr
     int *flag;
     const TMap *tmap;  // {h pairs, h rest, g pairs} of fin, or nullptr
@@ -168,6 +168,30 @@ __device__ __forceinline__ void rec_uni(T f0, T f1, T f2, T f3, T f4, T f5, T &r
     const T E0 = f0 - f3, E1 = f1 - f4, E2 = f2 - f5;
     rx = fma(T(2), E0, E1 - E2);
     ry = fma(T(2), E2, E1 - E0);
+}
+
+// Stress force of an interior node from the gradients at its neighbours (nb,
+// and their differences D_k across opposite ones); kka = kappa / (6h).  The
+// differences of the gradient products are formed in product form: P_k =
+// (E(d_x rho^2), E(d_y rho^2)), Q_k = E(d_x rho d_y rho); then
+// K_x = kappa [R_x(d_y rho^2) - R_y(d_x rho d_y rho)],
+// K_y = kappa [R_y(d_x rho^2) - R_x(d_x rho d_y rho)].
+template <typename T>
+__device__ __forceinline__ void stress_uni(V2<T> D0, V2<T> D1, V2<T> D2, const V2<T> *nb, T kka, T &kx, T &ky) {
+    V2<T> Pk[3];
+    T Qk[3];
+    auto prod = [&](int j, V2<T> D) {
+        const V2<T> u = nb[j], w = nb[j + 3];
+        Pk[j] = vmul(D, vadd(u, w));
+        Qk[j] = fma(u.x, D.y, w.y * D.x);
+    };
+    prod(0, D0);
+    prod(1, D1);
+    prod(2, D2);
+    const T rxy = fma(T(2), Pk[0].y, Pk[1].y - Pk[2].y), ryq = fma(T(2), Qk[2], Qk[1] - Qk[0]);
+    const T ryx = fma(T(2), Pk[2].x, Pk[1].x - Pk[0].x), rxq = fma(T(2), Qk[0], Qk[1] - Qk[2]);
+    kx = kka * (rxy - ryq);
+    ky = kka * (ryx - rxq);
 }
 
 // Whether the interior weights of a structured mesh are those of the split
@@ -906,26 +930,9 @@ __device__ __forceinline__ bool lat_tile_impl(const LatArgs<T> &A, const LatCoef
                    dmx, dmy);
         dmx *= A.al;
         dmy *= A.al;
-        // differences of the gradient products across opposite neighbours,
-        // in product form: (P.x, P.y) = E(d_x rho^2), E(d_y rho^2);
-        // Q = E(d_x rho d_y rho); then
-        // K_x = kappa [R_x(d_y rho^2) - R_y(d_x rho d_y rho)],
-        // K_y = kappa [R_y(d_x rho^2) - R_x(d_x rho d_y rho)]
-        V2<T> Pk[3];
-        T Qk[3];
-        auto prod = [&](int j, V2<T> u, V2<T> w) {
-            const V2<T> D = vsub<T>(u, w);
-            Pk[j] = vmul(D, vadd(u, w));
-            Qk[j] = fma(u.x, D.y, w.y * D.x);
-        };
-        prod(0, s_g[a2][b2 + 1], s_g[a2][b2 - 1]);
-        prod(1, s_g[a2 + 1][b2 + 1], s_g[a2 - 1][b2 - 1]);
-        prod(2, s_g[a2 + 1][b2], s_g[a2 - 1][b2]);
-        const T rxy = fma(T(2), Pk[0].y, Pk[1].y - Pk[2].y), ryq = fma(T(2), Qk[2], Qk[1] - Qk[0]);
-        const T ryx = fma(T(2), Pk[2].x, Pk[1].x - Pk[0].x), rxq = fma(T(2), Qk[0], Qk[1] - Qk[2]);
-        const T kka = P.kappa * A.al;
-        kx = kka * (rxy - ryq);
-        ky = kka * (ryx - rxq);
+        const V2<T> nb[6] = {s_g[a2][b2 + 1], s_g[a2 + 1][b2 + 1], s_g[a2 + 1][b2],
+                             s_g[a2][b2 - 1], s_g[a2 - 1][b2 - 1], s_g[a2 - 1][b2]};
+        stress_uni<T>(vsub<T>(nb[0], nb[3]), vsub<T>(nb[1], nb[4]), vsub<T>(nb[2], nb[5]), nb, P.kappa * A.al, kx, ky);
     } else {
         T smx = T(0), smy = T(0), skx = T(0), sky = T(0);
         const T mc = s_mu[ly + 1][lx + 1];

@@ -84,12 +84,12 @@ static bool encode_state(PFN_cuTensorMapEncodeTiled_v12000 fn, const felbm_state
 void lattice_tmaps(felbm_state *s) {
     s->d_tmap = nullptr;
     const felbm_mesh *m = s->mesh;
-    if (m->kind != 1 || m->sinfo.pitch % 4 != 0) return;
+    // (FP64 states step by passes over global fields, without boxes)
+    if (m->kind != 1 || m->sinfo.pitch % 4 != 0 || s->esize != 4) return;
     PFN_cuTensorMapEncodeTiled_v12000 fn = encoder();
     if (!fn) return;
     TMap maps[6];
-    const bool ok = s->esize == 8 ? encode_state<double>(fn, s, maps) : encode_state<float>(fn, s, maps);
-    if (!ok) return;
+    if (!encode_state<float>(fn, s, maps)) return;
     TMap *d = nullptr;
     if (cudaMalloc((void **)&d, sizeof(maps)) != cudaSuccess) {
         cudaGetLastError();
