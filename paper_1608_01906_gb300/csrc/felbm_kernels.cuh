@@ -298,9 +298,10 @@ __global__ void __launch_bounds__(256) k_mu_lap64(const __grid_constant__ Topo64
 // evaluated as psibar = psi* + (1 - w)(eq - psi*) + (1 + w) S: every rounding
 // then falls on the small collision increment instead of on O(w_a rho) terms
 // (in FP32 the other order repeats the same O(ulp(rho)) error every step).
-// With q = e.u + 3/2 (e.u)^2 - u.u/2 (so that Gamma_a - w_a = 3 w_a q and
-// 3 Gamma_a = 3 w_a (1 + 3 q)) and the forces scaled by (1 + w) dt/2 once per
-// node, the increments are
+// The sources of the two precisions are formed differently:
+// FP64 (its pipe bounds a step): with q = e.u + 3/2 (e.u)^2 - u.u/2 (so that
+// Gamma_a - w_a = 3 w_a q and 3 Gamma_a = 3 w_a (1 + 3 q)) and the forces
+// scaled by (1 + w) dt/2 once per node, the increments are
 //   h: -(1-w) (h* - rho w_a) + 3 w_a [c + q (m + 3 c)],
 //      c = (e-u).X, X = c_s^2 grad rho - rho grad mu, m = (1-w) rho;
 //   g: -(1-w) (g* - 3 w_a p) + 3 w_a [k + b + q (m + d + 3 k)],
@@ -308,7 +309,10 @@ __global__ void __launch_bounds__(256) k_mu_lap64(const __grid_constant__ Topo64
 //      (1+w) rho/2 [e.du + e.du (3 e.u + 3/2 e.du) - du.(2u + du)/2]:
 // two products per population with sums that are the node's but for the sign
 // of their odd part, 23 packed operations for a pair against 56 when each
-// term was formed by itself.
+// term is formed by itself (256 x 1024 Rayleigh-Taylor 423 -> 358 us a step).
+// FP32 forms each term by itself: there the products save 1.5 % of a lattice
+// step, and leave u twice as far from 64 bits (after 200 steps of a drop on
+// 57 x 103 nodes 9.4e-7 against 4.0e-7, on 32 x 32 7.3e-7 against 3.6e-7).
 template <typename T>
 struct CollidePrep {
     T r, ux, uy, p;
@@ -318,6 +322,10 @@ struct CollidePrep {
     T Vx, Vy, gA;     // grad rho + 3 K (scaled); even part m - u.V
     T Bx, By, gZ;     // K + G; even part -u.K - (1+w) rho/4 du.(2u + du)
     T Gx, Gy, dux, duy;  // (1+w) rho/2 du, and du
+};
+template <>
+struct CollidePrep<float> {
+    float r, ux, uy, p, omw, opw, hdt, Xx, Xy, uX, uD, uK, uu, dux, duy, udu, drx, dry, kx, ky;
 };
 
 // Correctly rounded reciprocal (the same value as T(1) / x).
@@ -337,28 +345,12 @@ __device__ __forceinline__ T div3(T x) {
     return fma(r, c, q);
 }
 
-// sg = sum_a g*_a, mx, my = sum_a e_a g*_a of the streamed (and bounced) g.
+// The scalars of the sources for given moments (omw = 1 - w, opw = 1 + w).
 template <typename T>
-__device__ __forceinline__ CollidePrep<T> collide_prep(const Phys<T> &P, T sg, T mx, T my, T r,
-                                                       T drx, T dry, T dmx, T dmy, T kx, T ky) {
+__device__ __forceinline__ void collide_terms(const Phys<T> &P, CollidePrep<T> &c, T omw, T opw, T drx, T dry, T dmx,
+                                              T dmy, T kx, T ky) {
     constexpr T cs2 = T(1) / T(3);
-    CollidePrep<T> c;
-    const T hdt = T(0.5) * P.dt;
-    const T inv_r = recip_rn(r);
-    c.r = r;
-    c.ux = (mx + hdt * kx + hdt * r * P.gx) * inv_r;
-    c.uy = (my + hdt * ky + hdt * r * P.gy) * inv_r;
-    // p = c_s^2 (...) as a division by 3: a rounded 1/3 would be a gain on p
-    // every step (see kW3)
-    c.p = div3(sg + hdt * (c.ux * drx + c.uy * dry));
-    T C = (r - P.rho_v) * P.inv_drho;
-    C = C < T(0) ? T(0) : (C > T(1) ? T(1) : C);
-    // 1/tau = C/tau_l + (1-C)/tau_v; w = (2 tau - 1)/(2 tau + 1) gives, with
-    // s = 1/tau, 1 - w = 2 s/(2 + s) and 1 + w = 4/(2 + s): one reciprocal
-    const T s = C * P.inv_tau_l + (T(1) - C) * P.inv_tau_v;
-    const T d = recip_rn(T(2) + s);
-    const T omw = T(2) * s * d, opw = T(4) * d;
-    const T f = opw * hdt, m = omw * r;
+    const T r = c.r, f = opw * (T(0.5) * P.dt), m = omw * r;
     c.nr = -r;
     c.np = -c.p;
     c.nomw = -omw;
@@ -380,6 +372,48 @@ __device__ __forceinline__ CollidePrep<T> collide_prep(const Phys<T> &P, T sg, T
     c.Bx = Kx + c.Gx;
     c.By = Ky + c.Gy;
     c.gZ = -(c.ux * Kx + c.uy * Ky) - (c.Gx * (c.ux + T(0.5) * c.dux) + c.Gy * (c.uy + T(0.5) * c.duy));
+}
+__device__ __forceinline__ void collide_terms(const Phys<float> &P, CollidePrep<float> &c, float omw, float opw,
+                                              float drx, float dry, float dmx, float dmy, float kx, float ky) {
+    constexpr float cs2 = 1.0f / 3.0f;
+    c.omw = omw;
+    c.opw = opw;
+    c.hdt = 0.5f * P.dt;
+    c.Xx = cs2 * drx - c.r * dmx;  // F: c_s^2 grad rho - rho grad mu
+    c.Xy = cs2 * dry - c.r * dmy;
+    c.uX = c.ux * c.Xx + c.uy * c.Xy;
+    c.uD = c.ux * drx + c.uy * dry;
+    c.uK = c.ux * kx + c.uy * ky;
+    c.uu = c.ux * c.ux + c.uy * c.uy;
+    c.dux = P.gx * P.dt;  // exact-difference du = g dt
+    c.duy = P.gy * P.dt;
+    c.udu = c.dux * (2.0f * c.ux + c.dux) + c.duy * (2.0f * c.uy + c.duy);
+    c.drx = drx;
+    c.dry = dry;
+    c.kx = kx;
+    c.ky = ky;
+}
+
+// sg = sum_a g*_a, mx, my = sum_a e_a g*_a of the streamed (and bounced) g.
+template <typename T>
+__device__ __forceinline__ CollidePrep<T> collide_prep(const Phys<T> &P, T sg, T mx, T my, T r,
+                                                       T drx, T dry, T dmx, T dmy, T kx, T ky) {
+    CollidePrep<T> c;
+    const T hdt = T(0.5) * P.dt;
+    const T inv_r = recip_rn(r);
+    c.r = r;
+    c.ux = (mx + hdt * kx + hdt * r * P.gx) * inv_r;
+    c.uy = (my + hdt * ky + hdt * r * P.gy) * inv_r;
+    // p = c_s^2 (...) as a division by 3: a rounded 1/3 would be a gain on p
+    // every step (see kW3)
+    c.p = div3(sg + hdt * (c.ux * drx + c.uy * dry));
+    T C = (r - P.rho_v) * P.inv_drho;
+    C = C < T(0) ? T(0) : (C > T(1) ? T(1) : C);
+    // 1/tau = C/tau_l + (1-C)/tau_v; w = (2 tau - 1)/(2 tau + 1) gives, with
+    // s = 1/tau, 1 - w = 2 s/(2 + s) and 1 + w = 4/(2 + s): one reciprocal
+    const T s = C * P.inv_tau_l + (T(1) - C) * P.inv_tau_v;
+    const T d = recip_rn(T(2) + s);
+    collide_terms(P, c, T(2) * s * d, T(4) * d, drx, dry, dmx, dmy, kx, ky);
     return c;
 }
 
@@ -409,11 +443,59 @@ __device__ __forceinline__ void collide_pair(const CollidePrep<T> &c, V2<T> hs, 
     const V2<T> hz = vfma(q, vset(c.hA + eA, c.hA - eA), vset(c.hZ + eX, c.hZ - eX));
     const V2<T> gz = vfma(q, vset(c.gA + eV, c.gA - eV), vset(ge + eB, ge - eB));
     const V2<T> w32 = vset(w3, w3), nomw = vset(c.nomw, c.nomw);
-    const V2<T> hd = vfma(nomw, vfma(vset(c.nr, c.nr), vset(wa, wa), hs), vmul(w32, hz));
-    const V2<T> gd = vfma(nomw, vfma(vset(c.np, c.np), w32, gs), vmul(w32, gz));
-    ho = vadd(hs, hd);
-    go = vadd(gs, gd);
+    ho = vadd(hs, vfma(nomw, vfma(vset(c.nr, c.nr), vset(wa, wa), hs), vmul(w32, hz)));
+    go = vadd(gs, vfma(nomw, vfma(vset(c.np, c.np), w32, gs), vmul(w32, gz)));
     ds = vadd(ds, vfma(hs, vset(T(-1), T(-1)), ho));
+}
+
+// What one pair (or the rest population) of FP32 takes from the directions'
+// products e.v of the node's vectors, eq and source by themselves.
+struct PairTerms {
+    float eu, eX, eD, eK, ed, uX, uD, uK, uu, udu, r, p, omw, opw, hdt;
+};
+__device__ __forceinline__ void collide_terms_pair(const PairTerms &t, float wa, float w3, float2 hs, float2 gs,
+                                                   float2 &ho, float2 &go) {
+    // Gamma - w = 3w (e.u + 1.5 (e.u)^2 - 0.5 u.u), formed without the w
+    // offset (keeps the momentum part); 3w from kW3
+    const float even = 1.5f * t.eu * t.eu - 0.5f * t.uu;
+    const float2 gmw = vfma(vset(w3, w3), vset(t.eu, -t.eu), vset(w3 * even, w3 * even));
+    const float2 gam3 = vfma(vset(3.0f, 3.0f), gmw, vset(w3, w3));  // 3 Gamma
+    const float2 Fa = vmul(vset(t.hdt * (t.eX - t.uX), t.hdt * (-t.eX - t.uX)), gam3);
+    const float2 Ga = vfma(vset(t.hdt * (t.eD - t.uD), t.hdt * (-t.eD - t.uD)), gmw,
+                           vmul(vset(t.hdt * (t.eK - t.uK), t.hdt * (-t.eK - t.uK)), gam3));
+    // 1/2 [g_eq(u + du) - g_eq(u)] = rho/2 [Gamma(u + du) - Gamma(u)]
+    const float bev = 1.5f * t.ed * (2.0f * t.eu + t.ed) - 0.5f * t.udu;
+    const float hrw = 0.5f * t.r * w3;
+    const float2 Sg = vfma(vset(hrw, hrw), vset(t.ed + bev, bev - t.ed), Ga);
+    const float2 rg = vmul(vset(t.r, t.r), gmw);
+    const float2 dh = vadd(vfma(vset(t.r, t.r), vset(wa, wa), vset(-hs.x, -hs.y)), rg);  // h_eq - h*
+    const float2 dg = vadd(vfma(vset(w3, w3), vset(t.p, t.p), vset(-gs.x, -gs.y)), rg);  // g_eq - g*
+    ho = vadd(hs, vfma(vset(t.omw, t.omw), dh, vmul(vset(t.opw, t.opw), Fa)));
+    go = vadd(gs, vfma(vset(t.omw, t.omw), dg, vmul(vset(t.opw, t.opw), Sg)));
+}
+__device__ __forceinline__ void collide_terms_rest(const PairTerms &t, float wa, float w3, float hs, float gs,
+                                                   float &ho, float &go) {
+    const float gmw = w3 * (-0.5f * t.uu), gam3 = w3 + 3.0f * gmw;
+    const float Fa = t.hdt * -t.uX * gam3;
+    const float Sg = t.hdt * -t.uD * gmw + t.hdt * -t.uK * gam3 + 0.5f * t.r * w3 * (-0.5f * t.udu);
+    const float dh = fma(t.r, wa, -hs) + t.r * gmw, dg = fma(w3, t.p, -gs) + t.r * gmw;
+    ho = hs + (t.omw * dh + t.opw * Fa);
+    go = gs + (t.omw * dg + t.opw * Sg);
+}
+template <int ex, int ey>
+__device__ __forceinline__ PairTerms pair_terms(const CollidePrep<float> &c) {
+    if (ex == 0 && ey == 0)
+        return {0.f, 0.f, 0.f, 0.f, 0.f, c.uX, c.uD, c.uK, c.uu, c.udu, c.r, c.p, c.omw, c.opw, c.hdt};
+    return {dir_dot<ex, ey>(c.ux, c.uy), dir_dot<ex, ey>(c.Xx, c.Xy), dir_dot<ex, ey>(c.drx, c.dry),
+            dir_dot<ex, ey>(c.kx, c.ky), dir_dot<ex, ey>(c.dux, c.duy), c.uX, c.uD, c.uK, c.uu, c.udu,
+            c.r, c.p, c.omw, c.opw, c.hdt};
+}
+template <typename T, int Q>
+__device__ __forceinline__ void collide_pair(const CollidePrep<float> &c, float2 hs, float2 gs, float2 &ho,
+                                             float2 &go, float2 &ds) {
+    constexpr int A = pair_dir(Q, 0);
+    collide_terms_pair(pair_terms<kEx(A), kEy(A)>(c), kW<float>(A), kW3<float>(A), hs, gs, ho, go);
+    ds = vadd(ds, vfma(hs, vset(-1.0f, -1.0f), ho));
 }
 
 // The same for the rest population; its h also takes the sum of the node's
@@ -423,9 +505,14 @@ __device__ __forceinline__ void collide_pair(const CollidePrep<T> &c, V2<T> hs, 
 template <typename T>
 __device__ __forceinline__ void collide_rest(const CollidePrep<T> &c, T hs, T gs, V2<T> ds, T &ho, T &go) {
     constexpr T wa = kW<T>(0), w3 = kW3<T>(0);
-    const T h = hs + fma(c.nomw, fma(c.nr, wa, hs), w3 * fma(c.nhuu, c.hA, c.hZ));
+    T h;
+    if constexpr (sizeof(T) == 4) {
+        collide_terms_rest(pair_terms<0, 0>(c), wa, w3, hs, gs, h, go);
+    } else {
+        h = hs + fma(c.nomw, fma(c.nr, wa, hs), w3 * fma(c.nhuu, c.hA, c.hZ));
+        go = gs + fma(c.nomw, fma(c.np, w3, gs), w3 * fma(c.nhuu, c.gA, c.gZ));
+    }
     ho = h - ((ds.x + ds.y) + (h - hs));
-    go = gs + fma(c.nomw, fma(c.np, w3, gs), w3 * fma(c.nhuu, c.gA, c.gZ));
 }
 
 // Zeroth and first moments of the streamed g.  The first moments are summed
