@@ -312,7 +312,7 @@ static void step_lattice(felbm_state *s, LatArgs<T> &A, bool write_mom) {
     A.tmap = s->d_tmap ? s->d_tmap + 3 * s->cur : nullptr;
     const dim3 grd((A.nx + kLTX - 1) / kLTX, (A.yhi - A.ylo + kLTY - 1) / kLTY);
     const int sl = prof_begin(s, 4);
-    k_lat_step<T, LAP64><<<grd, dim3(kLTX, kLTY), lat_smem<T>(), m->stream>>>(A);
+    launch_pdl(k_lat_step<T, LAP64>, grd, dim3(kLTX, kLTY), lat_smem<T>(), m->stream, A);
     prof_end(s, sl);
     s->cur ^= 1;
 }

@@ -126,14 +126,16 @@ __global__ void __launch_bounds__(kNT, (sizeof(T) == 4 ? 1024 : 512) / kNT) k_ba
     __shared__ StepSmem<T> S;
     __shared__ __align__(16) LatArgs<T> sA;
     extern __shared__ __align__(128) unsigned char bdsm[];
+    lat_block_init<T>(S);
+    // (what no kernel writes, before the wait)
+    const TileRef r = B.tiles[blockIdx.x];
+    int cur = -1;
+    load_mesh<T>(B, r.mesh, sA, cur);
+    pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
         B.ctr[0] = 0u;
         B.ctr[1] = 0u;
     }
-    lat_block_init<T>(S);
-    const TileRef r = B.tiles[blockIdx.x];
-    int cur = -1;
-    load_mesh<T>(B, r.mesh, sA, cur);
     TilePipe pp;
     const NextTile none{0, 0, 0, false, false};
     lat_tile<T>(sA, batch_coef<T, SC>(B, sA), r.bx, r.by, S, bdsm, pp, none);
@@ -255,9 +257,9 @@ static cudaError_t batch_launch32(felbm_batch *b, int parity, int write_mom) {
         else
             k_batch_step<float, false><<<grid, blk, sm, b->stream>>>(B);
     } else if (b->shared_coef) {
-        k_batch_tile<float, true><<<(unsigned)b->ntiles, blk, sm, b->stream>>>(B);
+        launch_pdl(k_batch_tile<float, true>, (unsigned)b->ntiles, blk, sm, b->stream, B);
     } else {
-        k_batch_tile<float, false><<<(unsigned)b->ntiles, blk, sm, b->stream>>>(B);
+        launch_pdl(k_batch_tile<float, false>, (unsigned)b->ntiles, blk, sm, b->stream, B);
     }
     return cudaGetLastError();
 }

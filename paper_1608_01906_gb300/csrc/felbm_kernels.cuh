@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (ONE ? 4 : 5) : 2)
     const auto row = m.row(i);
     const int k = m.tag_of(i);
     pdl_wait();
-    pdl_trigger();
+    if (ONE) pdl_trigger();
     V2<T> hp[4];
     stream_pairs<T>(m, f, np, i, dt, hp, [&](auto &&fn) { m.each(row, fn); });
     const size_t si = m.slot(i);
@@ -205,7 +205,6 @@ __global__ void __launch_bounds__(256) k_grad(const __grid_constant__ Topo m, Fi
     if (i >= m.n) return;
     const auto row = m.row(i);
     pdl_wait();
-    pdl_trigger();
     T gx, gy;
     recover(m, row, F.rho, i, gx, gy);
     F.drx[i] = gx;
@@ -246,7 +245,6 @@ __global__ void __launch_bounds__(256) k_mu(const __grid_constant__ Topo m, Fiel
     if (i >= m.n) return;
     const auto row = m.row(i);
     pdl_wait();
-    pdl_trigger();
     const T gxi = F.drx[i], gyi = F.dry[i];
     T lap = T(0), kx = T(0), ky = T(0);
     m.each(row, [&](int32_t j, T ax, T ay, T, T, T) {
@@ -271,7 +269,6 @@ __global__ void __launch_bounds__(256) k_mu_lap64(const __grid_constant__ Topo64
     if (i >= m.n) return;
     const auto row = m.row(i);
     pdl_wait();
-    pdl_trigger();
     const float gxi = F.drx[i], gyi = F.dry[i];
     double lap = 0.0;
     float kx = 0.f, ky = 0.f;
@@ -594,7 +591,6 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 2) k_collide(const _
     const auto row = m.row(i);
     const int k = m.tag_of(i);
     pdl_wait();
-    pdl_trigger();
     // g streamed here (the h code on the g half of the state); h* was
     // streamed and bounced back by k_rho
     T dmx, dmy;

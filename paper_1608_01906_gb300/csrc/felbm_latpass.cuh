@@ -197,7 +197,6 @@ __device__ __forceinline__ void lat_pass(const LatArgs<T> &A, int64_t idx) {
 template <typename T, int S>
 __global__ void __launch_bounds__(kPassBlock) k_lat_pass(const __grid_constant__ LatArgs<T> A) {
     pdl_wait();
-    pdl_trigger();
     lat_pass<T, S>(A, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 

@@ -703,7 +703,7 @@ __device__ __forceinline__ bool lat_tile_impl(const LatArgs<T> &A, const LatCoef
     const bool valid = INTERIOR || (x < nx && y < A.yhi);
     const int32_t i = valid ? x + nx * y : 0;                        // node (moments)
     const size_t ip = valid ? (size_t)x + (size_t)A.pitch * y : 0;  // population slot
-    const T g0 = valid ? __ldg(A.fin + 9 * np + ip) : T(0);
+    const T g0 = valid ? A.fin[9 * np + ip] : T(0);
     // rows of the rho region (y0 - 3 .. y0 + 10) all of kind 0 and inside
     // (decided on the whole lattice's rows: row y0 + row0 of gny)
     const bool rows_in = INTERIOR || !walls || (y0 + A.row0 >= kHD && y0 + A.row0 + kLTY + kHD <= A.gny);
@@ -1027,6 +1027,7 @@ __global__ void __launch_bounds__(kNT, (sizeof(T) == 4 ? 1024 : 512) / kNT) k_la
     __shared__ StepSmem<T> S;
     extern __shared__ __align__(128) unsigned char lat_dsm[];
     lat_block_init<T>(S);
+    pdl_wait();
     TilePipe pp;
     const NextTile none{0, 0, 0, false, false};
     lat_tile<T, LAP64>(A, A.c, blockIdx.x, blockIdx.y, S, lat_dsm, pp, none);

@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
     const auto row = m.template row<false>(g);
     const int tag = m.tag_of(g);
     pdl_wait();
-    pdl_trigger();
+    if (ONE) pdl_trigger();
     // rho of the region, in flight while g is streamed (the own rows' a from
     // shared memory, the rest of their entries from the mesh's rows)
     const T *grho = A.c.F.rho;
