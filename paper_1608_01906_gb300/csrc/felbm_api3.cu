@@ -94,6 +94,7 @@ static DevLattice3<T> dev_lat3(const felbm_mesh *m, double dt) {
             }
             for (int c = 0; c < 3; ++c) d.k.a[k][o][c] = (T)cf[c];
         }
+    d.k.s12 = (T)(L.c[0][0][0] / kuhn_w(0, 0));
     return d;
 }
 
@@ -128,16 +129,54 @@ static Fields3<T> fields3_of(felbm_state *s) {
     return F;
 }
 
+// Forms of the passes over a lattice (us a launch or step, GB300):
+//   streaming of h split over four threads a node up to 2^16 nodes (FP32 step
+//   of 32^3 14.0 us split, 15.9 with a thread per node; 40^3 20.5 and 22.0;
+//   48^3 26.0 and 25.2; FP64 pass 24^3 29 and 47, 36^3 58 and 87, 48^3 130
+//   and 127), a thread per node above;
+//   the collision likewise in FP64 (14^3 30 and 46, 36^3 117 and 125, 48^3
+//   265 and 244); in FP32 always a thread per node (16^3 9.9 us a step
+//   against 9.6 split, 32^3 14.0 and 15.0, 64^3 42.9 and 57);
+//   the scalar passes with two nodes a column from 2^18 nodes on in FP32
+//   (96^3 26.4 us for the two, 30.2 with one; 64^3 equal), else one.
+constexpr int64_t kSplitMax = 1 << 16, kColumnMin = 1 << 18;
+
+template <typename T, typename Fn>
+static void with_lz(const DevLattice3<T> &d, Fn &&fn) {
+    if constexpr (sizeof(T) == 4) {
+        if (d.n >= kColumnMin) return fn(std::integral_constant<int, 2>());
+    }
+    fn(std::integral_constant<int, 1>());
+}
+
+template <typename T>
+static unsigned col_grid(const DevLattice3<T> &d, int lz) {
+    return nblocks3((int64_t)d.nx * d.ny, 256) * nblocks3(d.nz, lz);
+}
+
 // grad rho, then lap rho, K and mu, from F.rho.
 template <typename T, typename Topo>
 static void chain3(felbm_state *s, const Topo &d, const Fields3<T> &F, const Phys3<T> &P) {
     const felbm_mesh *m = s->mesh;
-    const unsigned g = nblocks3(m->n_nodes, 256);
     int sl = prof_begin(s, 1);
-    k_grad3<T, Topo><<<g, 256, 0, m->stream>>>(d, F);
+    if constexpr (Topo::kLattice) {
+        with_lz<T>(d, [&](auto Z) {
+            constexpr int LZ = decltype(Z)::value;
+            launch_pdl(k_grad3_col<T, LZ>, col_grid(d, LZ), 256, 0, m->stream, d, F);
+        });
+    } else {
+        launch_pdl(k_grad3_rows<T>, nblocks3(m->n_nodes, kSplitNodes), kSplitBlock, 0, m->stream, d, F);
+    }
     prof_end(s, sl);
     sl = prof_begin(s, 2);
-    k_mu3<T, Topo><<<g, 256, 0, m->stream>>>(d, F, P);
+    if constexpr (Topo::kLattice) {
+        with_lz<T>(d, [&](auto Z) {
+            constexpr int LZ = decltype(Z)::value;
+            launch_pdl(k_mu3_col<T, LZ>, col_grid(d, LZ), 256, 0, m->stream, d, F, P);
+        });
+    } else {
+        launch_pdl(k_mu3_rows<T>, nblocks3(m->n_nodes, kSplitNodes), kSplitBlock, 0, m->stream, d, F, P);
+    }
     prof_end(s, sl);
 }
 
@@ -169,8 +208,13 @@ static void step3(felbm_state *s, const Topo &d, const Fields3<T> &F, const Phys
     const felbm_mesh *m = s->mesh;
     const T *fin = reinterpret_cast<const T *>(s->f[s->cur]);
     T *fout = reinterpret_cast<T *>(s->f[s->cur ^ 1]);
+    const bool split = !Topo::kLattice || d.n <= kSplitMax;
     int sl = prof_begin(s, 0);
-    k_rho3<T, Topo><<<nblocks3(m->n_nodes, 256), 256, 0, m->stream>>>(d, fin, P.dt, F.rho, F.hs);
+    if (split)
+        launch_pdl(k_rho3_split<T, Topo>, nblocks3(m->n_nodes, kSplitNodes), kSplitBlock, 0, m->stream, d, fin, P.dt,
+                   F.rho, F.hs);
+    else if constexpr (Topo::kLattice)
+        launch_pdl(k_rho3_node<T>, nblocks3(m->n_nodes, 256), 256, 0, m->stream, d, fin, P.dt, F.rho, F.hs);
     prof_end(s, sl);
     chain3<T>(s, d, F, P);
     Collide3Args<T, Topo> A;
@@ -182,7 +226,14 @@ static void step3(felbm_state *s, const Topo &d, const Fields3<T> &F, const Phys
     A.mom = write_mom ? reinterpret_cast<T *>(s->mom) : nullptr;
     A.flag = s->d_flag;
     sl = prof_begin(s, 3);
-    k_collide3<T, Topo><<<nblocks3(m->n_nodes, 128), 128, 0, m->stream>>>(A);
+    if constexpr (Topo::kLattice) {
+        if (sizeof(T) == 4 || !split)
+            launch_pdl(k_collide3_node<T>, nblocks3(m->n_nodes, 128), 128, 0, m->stream, A);
+        else if constexpr (sizeof(T) == 8)
+            launch_pdl(k_collide3_split<T, Topo>, nblocks3(m->n_nodes, kSplitNodes), kSplitBlock, 0, m->stream, A);
+    } else {
+        launch_pdl(k_collide3_split<T, Topo>, nblocks3(m->n_nodes, kSplitNodes), kSplitBlock, 0, m->stream, A);
+    }
     prof_end(s, sl);
     s->cur ^= 1;
 }
