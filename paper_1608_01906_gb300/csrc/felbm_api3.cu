@@ -130,13 +130,13 @@ static Fields3<T> fields3_of(felbm_state *s) {
 }
 
 // Forms of the passes over a lattice (us a launch or step, GB300):
-//   streaming of h split over four threads a node up to 2^16 nodes (FP32 step
-//   of 32^3 14.0 us split, 15.9 with a thread per node; 40^3 20.5 and 22.0;
-//   48^3 26.0 and 25.2; FP64 pass 24^3 29 and 47, 36^3 58 and 87, 48^3 130
-//   and 127), a thread per node above;
+//   streaming of h split over three threads a node up to 2^16 nodes (FP32
+//   step of 32^3 12.1 us split, 13.4 with a thread per node; 40^3 17.5 and
+//   18.0; 48^3 26.0 and 25.2; FP64 pass 24^3 27 and 47, 36^3 58 and 87, 48^3
+//   130 and 127), a thread per node above;
 //   the collision likewise in FP64 (14^3 30 and 46, 36^3 117 and 125, 48^3
 //   265 and 244); in FP32 always a thread per node (16^3 9.9 us a step
-//   against 9.6 split, 32^3 14.0 and 15.0, 64^3 42.9 and 57);
+//   against 9.2 split, 24^3 11.0 and 11.6, 64^3 42.9 and 57);
 //   the scalar passes with two nodes a column from 2^18 nodes on in FP32
 //   (96^3 26.4 us for the two, 30.2 with one; 64^3 equal), else one.
 constexpr int64_t kSplitMax = 1 << 16, kColumnMin = 1 << 18;

@@ -12,9 +12,9 @@
 //   collide   recovered grad mu, streaming of the 19 g populations,
 //             bounce-back, moments (Eqs. velocity, pressure) and the
 //             post- and next pre-streaming collision (Sec. 2.2).
-// Each pass has a form that splits a node over four threads (k_*3_split, or
-// k_*3_rows: general meshes, small lattices) and one in which a thread has a
-// column of nodes of the lattice (k_*3_col).
+// Each pass has a form that splits a node over three threads (k_*3_split or
+// k_*3_rows: general meshes, small lattices) and one for lattices with a
+// thread per node (k_*3_node) or per column of nodes (k_*3_col).
 // D3Q19 directions are ordered so that 2q+1 and 2q+2 are opposite (q =
 // 0..8); the populations are stored as the rest value plus 9 interleaved
 // opposite pairs (pop layout of felbm_internal.h with 19 per distribution).
@@ -338,6 +338,11 @@ __device__ __forceinline__ void bounce_pair3(int k, int q, V2<T> &p) {
 }
 
 // ---- a thread per node: large lattices ---------------------------------------
+// Bound by the latency of the gathers at 32 (h) and 20 (g) warps an SM and, from
+// 10^6 nodes on, by HBM with the h* round trip (128^3 FP32: 111 and 169 us for
+// 327 and 713 MB).  All pairs of a neighbour at once is the order that hides
+// most: pair by pair over columns of 1, 2 or 4 nodes, which loads 11 or 9
+// values a node and pair instead of 15, took 142, 132 and 183 us for h.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1)
     k_rho3_node(const __grid_constant__ DevLattice3<T> m, const T *f, T dt, T *rho, T *hs) {
@@ -364,17 +369,19 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1)
     hs[i] = h0;
 }
 
-// ---- a node split over four threads ----------------------------------------
-// A block has 64 nodes; the warps 2 g and 2 g + 1 of it take the pairs of
-// group g (pairs 0-2, 3-4, 5-6, 7-8).  The groups of a node read its row one
-// after the other, from L1.  What bounds the passes below some 10^5 nodes is
-// the latency of the gathers (14 neighbours x 9 pairs, two accesses deep on
-// general rows); a thread per node has 13 warps per SM on a 40^3 mesh, four
-// have 53 and a third of the registers.
+// ---- a node split over three threads -----------------------------------------
+// A block has 64 nodes; the warps 2 g and 2 g + 1 of it take the pairs 3 g ..
+// 3 g + 2.  The groups of a node read its row one after the other, from L1.
+// What bounds the passes below some 10^5 nodes is the latency of the gathers
+// (14 neighbours x 9 pairs, two accesses deep on general rows); a thread per
+// node has 13 warps per SM on a 40^3 mesh, three have 40 and each waits for a
+// third of the gathers.  Jittered tetrahedra, FP32, us a step: 40^3 52 -> 37.8,
+// 16^3 15.3; four threads (3, 2, 2, 2 pairs) 39.2 and 15.4, with more loads of
+// the rows.
 constexpr int kSplitNodes = 64;
 constexpr int kSplitBlock = kSplitNodes * kSplitGroups;
-constexpr int split_first(int g) { return kSplitGroups == 3 ? 3 * g : (g == 0 ? 0 : 1 + 2 * g); }
-constexpr int split_count(int g) { return kSplitGroups == 3 || g == 0 ? 3 : 2; }
+constexpr int split_first(int g) { return 3 * g; }
+constexpr int split_count(int) { return 3; }
 
 // Runs fn(integral_constant<g>) with the group of the thread (warp-uniform).
 template <typename Fn>
@@ -383,10 +390,8 @@ __device__ __forceinline__ void by_group(int g, Fn &&fn) {
         fn(std::integral_constant<int, 0>());
     else if (g == 1)
         fn(std::integral_constant<int, 1>());
-    else if (kSplitGroups == 3 || g == 2)
-        fn(std::integral_constant<int, 2>());
     else
-        fn(std::integral_constant<int, kSplitGroups - 1>());
+        fn(std::integral_constant<int, 2>());
 }
 
 // The sum of the groups' values of a node.
@@ -437,9 +442,10 @@ __global__ void __launch_bounds__(kSplitBlock, sizeof(T) == 4 ? 4 : 2)
 
 // ---- columns of the lattice --------------------------------------------------
 // A thread has LZ nodes one above the other.  The 14 neighbours of a node lie
-// at 7 places of its plane, 4 above and 4 below, and a column shares them:
-// 11 loads a node and value for LZ = 2, 9 for LZ = 4, against 15; a block's
-// rows of a plane are read from L2 once for all its planes.
+// at 7 places of its plane, 4 above and 4 below, and a column shares them: 11
+// loads a node for LZ = 2 against 15.  The scalar passes (grad rho; mu and K)
+// with the integer weights, us on 128^3 FP32: 21.0 and 47.0 with the tables,
+// 19 and 36 with LZ = 1, 14.2 and 30.8 with LZ = 2; LZ = 4 no faster (14.4, 32).
 template <int LZ>
 struct Col3 {
     int32_t r[7];        // in the plane: own, +x, -x, +y, -y, +x+y, -x-y
@@ -538,8 +544,8 @@ __device__ __forceinline__ void mu_edge3(const T *cf, const T *gi, const T *gj, 
 }
 
 // ---- grad rho, mu and K -------------------------------------------------------
-// General rows, four threads a node: thread group g of a block (as in the
-// split passes) takes the entries g, g + 4, ... of the rows of its nodes, all
+// General rows, three threads a node: thread group g of a block (as in the
+// split passes) takes the entries g, g + 3, ... of the rows of its nodes, all
 // of them in flight at once, and the sums meet in shared memory.
 template <typename T, int NV>
 __device__ __forceinline__ void split_sum(T (&part)[NV][kSplitGroups][kSplitNodes], int grp, int l, T *v) {
