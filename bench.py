@@ -591,7 +591,7 @@ def main():
                             "step over the summed launch times" % len(per_step))
         roofline["kernel_share"] = 1.0
         roofline["largest_launch"] = {"kernel": dom_single, "share": dom_share}
-    if args.precision == "fp64" and not multi:
+    if args.precision == "fp64" and (not multi or kind == 1):
         tf = FP64_ALGO_FLOPS_PER_NODE * prob.n_nodes / (dom_avg_ms * 1e-3) / 1e12
         p64 = alu.get("fp64") or FP64_PEAK_TFLOPS
         roofline = {"bound": "alu", "achieved": tf, "peak": p64, "unit": "TFLOP/s",
@@ -631,7 +631,7 @@ def main():
                 "steps": args.fp64_steps, "ms_per_step": ms64 / args.fp64_steps, "dtype": "f64",
                 "kernel": "+".join(per64), "kernel_ms": k64_ms,
                 "hbm": {"achieved": hbm64, "peak": peak, "unit": "GB/s", "frac": hbm64 / peak}}
-        if dim == 2 and len(per64) == 1:
+        if dim == 2 and (len(per64) == 1 or kind == 1):
             tf = FP64_ALGO_FLOPS_PER_NODE * prob.n_nodes / (k64_ms * 1e-3) / 1e12
             pk = alu.get("fp64") or FP64_PEAK_TFLOPS
             fp64["roofline"] = {"bound": "alu", "achieved": tf, "peak": pk, "unit": "TFLOP/s",
