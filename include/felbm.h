@@ -168,7 +168,7 @@ int felbm_mesh_create_tet(const double *xyz, int64_t n_nodes, const int32_t *tet
                           void *stream, felbm_mesh **out);
 
 /* Mesh facts.  Any output pointer may be NULL.  kind: 0 = general
- * (unstructured CSR kernels), 1 = structured lattice, 2 = tetrahedral,
+ * (unstructured kernels), 1 = structured lattice, 2 = tetrahedral,
  * 3 = Kuhn tetrahedral lattice (n_tri then counts tetrahedra).  device_bytes: device memory held by the
  * mesh. */
 int felbm_mesh_info(const felbm_mesh *mesh, int64_t *n_nodes, int64_t *n_tri, int32_t *kind,
@@ -241,7 +241,7 @@ void felbm_state_destroy(felbm_state *state);
 /* ---- batched launch (many runs per launch; the paper has a single run) ---
  * A batch advances many states on structured meshes (felbm_mesh_info kind
  * 1) of any sizes in one launch per time step over every 32 x 8 tile of every
- * mesh.  Each state's results are the same as from felbm_step alone (same
+ * mesh (FP64: the four passes of a lattice step over all meshes).  Each state's results are the same as from felbm_step alone (same
  * per-tile code).  Step pairs are replayed from a CUDA graph.  With
  * FELBM_BATCH_AUTOTUNE the first felbm_batch_step long enough to afford it
  * times real steps under each candidate (a persistent grid of 1 to the
@@ -272,8 +272,9 @@ void felbm_batch_destroy(felbm_batch *batch);
 /* ---- profiling aid (no counterpart in the paper) ------------------------
  * Kernel kinds issued by felbm_step, reported by felbm_profile_read:
  *   0 stream h + rho, 1 grad rho, 2 lap rho / stress / mu,
- *   3 grad mu + stream + collide (the general four-pass step),
- *   4 lattice step (one launch per step on structured meshes),
+ *   3 grad mu + stream + collide (the four-pass steps: general, FP64 lattices,
+ *     tetrahedra),
+ *   4 lattice step (one launch per step on structured meshes in FP32),
  *   5 patch step (second launch per step on general triangle meshes, after 0),
  *   6-7 unused. */
 #define FELBM_PROFILE_KINDS 8
@@ -400,7 +401,7 @@ int felbm_slab_exchange(felbm_state *const *slabs, int32_t n_slabs);
 
 /* Checked build (library compiled with FELBM_CHECKED, libfelbm_checked.so):
  * the kernels bounds-check the indices they gather with -- node and slot
- * indices of the CSR, lattice and patch neighbours, shared-memory region
+ * indices of the general rows, lattice and patch neighbours, shared-memory region
  * indices, the cp.async fill plans, the TMA boxes' 16-byte x rule, the slab
  * halo copies -- and, instead of an out-of-range access, skip it and record
  * a bit of a device status word (no assert, no trap).  This call waits for

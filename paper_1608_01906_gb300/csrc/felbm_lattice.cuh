@@ -1,5 +1,6 @@
 // Structured-lattice step: one launch per time step, one 32 x 8 tile of
-// nodes per block (k_lat_step).
+// nodes per block (k_lat_step, FP32; FP64 lattices take the passes of
+// felbm_latpass.cuh, which share the operators below).
 //
 //   1. the 4 h pair tiles (halo depth 4) and the h rest tile are staged in
 //      shared memory; the h populations are streamed (Taylor-Galerkin,
