@@ -70,6 +70,18 @@ static cudaError_t upload_ell3(felbm_mesh *m, const std::vector<int32_t> &sb) {
     return e;
 }
 
+// Whether the interior recovery weights of a lattice are those of the full
+// split that the integer-weight passes assume, to 1e-12 of their size.
+static bool kuhn_uniform(const Lattice3Info &L) {
+    const double s12 = L.c[0][0][0] / kuhn_w(0, 0);
+    for (int o = 0; o < 14; ++o)
+        for (int c = 0; c < 3; ++c) {
+            const double w = (o % 2 ? -1.0 : 1.0) * kuhn_w(o / 2, c) * s12;
+            if (!(std::fabs(L.c[0][o][c] - w) <= 1e-12 * std::fabs(3.0 * s12))) return false;
+        }
+    return true;
+}
+
 template <typename T>
 static DevLattice3<T> dev_lat3(const felbm_mesh *m, double dt) {
     const Lattice3Info &L = m->linfo3;
@@ -95,6 +107,7 @@ static DevLattice3<T> dev_lat3(const felbm_mesh *m, double dt) {
             for (int c = 0; c < 3; ++c) d.k.a[k][o][c] = (T)cf[c];
         }
     d.k.s12 = (T)(L.c[0][0][0] / kuhn_w(0, 0));
+    d.uni = kuhn_uniform(L) ? 1 : 0;
     return d;
 }
 

@@ -174,7 +174,7 @@ template <typename T>
 struct Lat3Coef {
     V2<T> pc[3][14][9];
     T a[3][14][3];
-    T s12;  // 1 / (12 h): a = kuhn_w s12 in the interior
+    T s12;  // 1 / (12 h): a = kuhn_w s12 in the interior of a uniform lattice
 };
 
 // Kuhn-split cube lattice in natural order (i = x + nx (y + ny z)): the 14
@@ -185,6 +185,7 @@ struct DevLattice3 {
     static constexpr bool kLattice = true;
     int32_t n, nx, ny, nz;
     int32_t walls;
+    int32_t uni;  // the interior recovery weights are the integers kuhn_w times k.s12 (see kuhn_uniform)
     Lat3Coef<T> k;
 #ifdef __CUDACC__
     __device__ __forceinline__ int kind_of(int32_t i) const {
@@ -452,7 +453,7 @@ struct Col3 {
     int32_t pl[LZ + 2];  // first nodes of the planes z0 - 1 .. z0 + LZ (wrapped)
     int32_t z0, n;
     int count;           // nodes of the column in the lattice
-    bool wall;           // it has nodes of a wall layer
+    bool table;          // its nodes take the tables: some are of a wall layer, or the lattice is not uniform
     // false: no column of the lattice
     template <typename T>
     __device__ __forceinline__ bool set(const DevLattice3<T> &m) {
@@ -478,7 +479,7 @@ struct Col3 {
             z = z + 1 == m.nz ? 0 : z + 1;
         }
         count = m.nz - z0 < LZ ? m.nz - z0 : LZ;
-        wall = m.walls && (z0 == 0 || z0 + LZ >= m.nz);
+        table = !m.uni || (m.walls && (z0 == 0 || z0 + LZ >= m.nz));
         return true;
     }
     // node l of the column
@@ -608,10 +609,13 @@ __global__ void __launch_bounds__(kSplitBlock) k_mu3_rows(const __grid_constant_
     }
 }
 
-// Interior lattice nodes: 12 h a_ij are small integers, opposite at opposite
+// Interior nodes of a uniform lattice: 12 h a_ij are small integers, opposite at opposite
 // offsets, so that R f = (1/(12 h)) sum over the seven offset pairs p of
 // kuhn_w(p) (f_{+o} - f_{-o}), o = lat3_d*(2p).  Half the differences and
-// products of the table form, and weights without rounding.
+// products of the table form, and weights without rounding.  The host checks
+// the assembled weights against them (kuhn_uniform): elements that leave gaps
+// or cover the box unevenly, but alike around every node, are a lattice of
+// the same offsets with other weights, and take the tables.
 __host__ __device__ constexpr int kuhn_w(int p, int c) {
     return p < 3 ? (p == c ? 3 : -1) : (p < 6 ? (c == 5 - p ? -1 : 1) : 1);
 }
@@ -662,7 +666,7 @@ __global__ void __launch_bounds__(256) k_grad3_col(const __grid_constant__ DevLa
     if (!c.set(m)) return;
     pdl_wait();
     const T *rho = pdl_ptr(F.rho);
-    if (c.wall) {
+    if (c.table) {
         for (int l = 0; l < c.count; ++l) {
             const int32_t i = c.r[0] + (c.z0 + l) * m.nx * m.ny;
             T g[3];
@@ -689,7 +693,7 @@ __global__ void __launch_bounds__(256) k_mu3_col(const __grid_constant__ DevLatt
     if (!c.set(m)) return;
     pdl_wait();
     const T *dr4 = pdl_ptr(F.dr4), *rho = pdl_ptr(F.rho);
-    if (c.wall) {
+    if (c.table) {
         for (int l = 0; l < c.count; ++l) {
             const int32_t i = c.r[0] + (c.z0 + l) * m.nx * m.ny;
             T gi[3], lap = T(0), K[3] = {T(0), T(0), T(0)};
@@ -1070,7 +1074,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 1)
     T dm[3];
     V2<T> hp[9], gp[9];
     by_kind(m, i, [&](auto K) {
-        if (decltype(K)::value == 0)
+        if (decltype(K)::value == 0 && m.uni)
             kuhn_recover_node<T>(m, mu, i, dm);
         else
             recover3<T, decltype(K)::value>(m, mu, i, dm);
