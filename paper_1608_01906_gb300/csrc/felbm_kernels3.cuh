@@ -447,7 +447,11 @@ __global__ void __launch_bounds__(kSplitBlock, sizeof(T) == 4 ? 4 : 2)
 // loads a node for LZ = 2 against 15.  The scalar passes (grad rho; mu and K)
 // with the integer weights, us on 128^3 FP32: 21.0 and 47.0 with the tables,
 // 19 and 36 with LZ = 1, 14.2 and 30.8 with LZ = 2; LZ = 4 no faster (14.4, 32).
-template <int LZ>
+// A block takes columns of one layer of columns, whose plane offsets are then
+// the block's; PACK: columns in order, so that small planes share a block (3 x
+// 3 x 40000 FP32 122 us a step without, 67 with; 64^3 43.2 and 43.6, 12^3 FP64
+// 53 and 58, 3 x 3 x 1000 12.3 and 11.0).
+template <int LZ, bool PACK>
 struct Col3 {
     int32_t r[7];        // in the plane: own, +x, -x, +y, -y, +x+y, -x-y
     int32_t pl[LZ + 2];  // first nodes of the planes z0 - 1 .. z0 + LZ (wrapped)
@@ -457,9 +461,19 @@ struct Col3 {
     // false: no column of the lattice
     template <typename T>
     __device__ __forceinline__ bool set(const DevLattice3<T> &m) {
-        const int32_t L = m.nx * m.ny, planes = (L + blockDim.x - 1) / blockDim.x;  // blocks of LZ planes
-        const int32_t zb = blockIdx.x / planes, p = (blockIdx.x - zb * planes) * blockDim.x + threadIdx.x;
-        if (p >= L) return false;
+        const int32_t L = m.nx * m.ny;
+        int32_t zb, p;
+        if (PACK) {
+            const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;  // below 2^31 + 256
+            zb = k / L;
+            p = k - (uint32_t)zb * L;
+            if (zb >= (m.nz + LZ - 1) / LZ) return false;
+        } else {
+            const int32_t planes = (L + blockDim.x - 1) / blockDim.x;  // blocks of LZ planes
+            zb = blockIdx.x / planes;
+            p = (blockIdx.x - zb * planes) * blockDim.x + threadIdx.x;
+            if (p >= L) return false;
+        }
         const int32_t y = p / m.nx, x = p - y * m.nx;
         const int32_t xp = x == m.nx - 1 ? 1 - m.nx : 1, xm = x == 0 ? m.nx - 1 : -1;
         const int32_t yp = (y == m.ny - 1 ? 1 - m.ny : 1) * m.nx, ym = (y == 0 ? m.ny - 1 : -1) * m.nx;
@@ -644,8 +658,8 @@ __device__ __forceinline__ void kuhn_recover_node(const DevLattice3<T> &m, const
 }
 
 // Recovered gradients of a scalar at the nodes of an interior column.
-template <typename T, int LZ>
-__device__ __forceinline__ void recover_col3(const DevLattice3<T> &m, const Col3<LZ> &c, const T *f, T (&g)[LZ][3]) {
+template <typename T, int LZ, bool PACK>
+__device__ __forceinline__ void recover_col3(const DevLattice3<T> &m, const Col3<LZ, PACK> &c, const T *f, T (&g)[LZ][3]) {
     T v[LZ + 2][7];
     c.load(v, [&](int32_t j) { return ldp(f + j); });
 #pragma unroll
@@ -660,9 +674,9 @@ __device__ __forceinline__ void recover_col3(const DevLattice3<T> &m, const Col3
     }
 }
 
-template <typename T, int LZ>
+template <typename T, int LZ, bool PACK>
 __global__ void __launch_bounds__(256) k_grad3_col(const __grid_constant__ DevLattice3<T> m, Fields3<T> F) {
-    Col3<LZ> c;
+    Col3<LZ, PACK> c;
     if (!c.set(m)) return;
     pdl_wait();
     const T *rho = pdl_ptr(F.rho);
@@ -676,7 +690,7 @@ __global__ void __launch_bounds__(256) k_grad3_col(const __grid_constant__ DevLa
         return;
     }
     T g[LZ][3];
-    recover_col3<T, LZ>(m, c, rho, g);
+    recover_col3<T>(m, c, rho, g);
 #pragma unroll
     for (int l = 0; l < LZ; ++l)
         if (l < c.count) store_grad3<T>(F.dr4, c.id(l), g[l]);
@@ -687,9 +701,9 @@ struct Vec3 {
     T v[3];
 };
 
-template <typename T, int LZ>
+template <typename T, int LZ, bool PACK>
 __global__ void __launch_bounds__(256) k_mu3_col(const __grid_constant__ DevLattice3<T> m, Fields3<T> F, Phys3<T> P) {
-    Col3<LZ> c;
+    Col3<LZ, PACK> c;
     if (!c.set(m)) return;
     pdl_wait();
     const T *dr4 = pdl_ptr(F.dr4), *rho = pdl_ptr(F.rho);
