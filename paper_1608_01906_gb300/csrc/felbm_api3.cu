@@ -247,7 +247,8 @@ static void step3(felbm_state *s, const Topo &d, const Fields3<T> &F, const Phys
     sl = prof_begin(s, 3);
     if constexpr (Topo::kLattice) {
         if (sizeof(T) == 4 || !split)
-            launch_pdl(k_collide3_node<T>, nblocks3(m->n_nodes, 128), 128, 0, m->stream, A);
+            launch_pdl(d.uni ? k_collide3_node<T, true> : k_collide3_node<T, false>, nblocks3(m->n_nodes, 128), 128, 0,
+                       m->stream, A);
         else if constexpr (sizeof(T) == 8)
             launch_pdl(k_collide3_split<T, Topo>, nblocks3(m->n_nodes, kSplitNodes), kSplitBlock, 0, m->stream, A);
     } else {

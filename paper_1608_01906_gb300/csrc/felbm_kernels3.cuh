@@ -1075,7 +1075,8 @@ __global__ void __launch_bounds__(kSplitBlock, sizeof(T) == 4 ? 4 : 2)
 
 // (all loads before the first store: interleaved with them the pass took
 // 232 us, not 172, on a 128^3 lattice in FP32)
-template <typename T>
+// UNI: the lattice's uni (read here instead it cost 1 % of a step).
+template <typename T, bool UNI>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 1)
     k_collide3_node(const __grid_constant__ Collide3Args<T, DevLattice3<T>> A) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1088,7 +1089,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 1)
     T dm[3];
     V2<T> hp[9], gp[9];
     by_kind(m, i, [&](auto K) {
-        if (decltype(K)::value == 0 && m.uni)
+        if (decltype(K)::value == 0 && UNI)
             kuhn_recover_node<T>(m, mu, i, dm);
         else
             recover3<T, decltype(K)::value>(m, mu, i, dm);
