@@ -68,7 +68,7 @@ def parse():
     ap.add_argument("--split-step", action="store_true",
                     help="general triangle meshes: always the four-launch step")
     ap.add_argument("--patch-step", action="store_true",
-                    help="general triangle meshes: the two-launch patch step (the default)")
+                    help="general triangle meshes: always the two-launch patch step")
     ap.add_argument("--general", action="store_true",
                     help="force the general CSR kernels on a structured mesh")
     ap.add_argument("--serve-requests", type=int, default=40)

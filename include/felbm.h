@@ -64,7 +64,7 @@ typedef enum felbm_status {
 #define FELBM_MESH_GENERAL 0x4u /* never use the structured-lattice kernels */
 #define FELBM_PERIODIC_Z 0x8u   /* tetrahedral meshes: box[2] > 0 is the period in z */
 #define FELBM_MESH_SPLIT_STEP 0x10u /* general triangle meshes: always four launches per step */
-#define FELBM_MESH_PATCH_STEP 0x20u /* general triangle meshes: the two-launch patch step (the default) */
+#define FELBM_MESH_PATCH_STEP 0x20u /* general triangle meshes: always the two-launch patch step */
 
 /* precision of the stored distributions and of the bulk arithmetic */
 #define FELBM_FP64 0
@@ -118,11 +118,14 @@ typedef struct felbm_params {
  * The library computes element geometry, the lumped mass, the assembled
  * streaming/recovery coefficients and an internal node order: patches of
  * 256 nodes along a Hilbert curve over the domain, reverse Cuthill-McKee
- * order within a patch.  A general mesh steps in two launches per step: the
+ * order within a patch.  A general mesh steps in two launches per step (the
  * streamed h and rho, then one block per patch with the patch's nodes up to
- * 3 edges away staged in shared memory.  FELBM_MESH_SPLIT_STEP asks for four
- * launches per step over global fields instead (as does a mesh whose patches
- * do not fit shared memory); both give the same results bit for bit.  A mesh that is the structured split of a unit lattice
+ * 3 edges away staged in shared memory) or in four over global fields: FP32
+ * states take two, those with FP64 coefficients (FP64, FELBM_PARAM_LAP_FP64)
+ * two up to 77,824 nodes.  FELBM_MESH_PATCH_STEP and FELBM_MESH_SPLIT_STEP
+ * force one of the two (a mesh whose patches do not fit shared memory takes
+ * four launches all the same); both give the same results bit for bit.
+ * A mesh that is the structured split of a unit lattice
  * (node i at ((i mod nx) h, (i div nx) h), each square cut along its
  * (i,j)-(i+1,j+1) diagonal, periodic in x, periodic or walled in y) is served
  * by the structured-lattice kernels unless FELBM_MESH_GENERAL is set.

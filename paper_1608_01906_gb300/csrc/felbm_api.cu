@@ -407,10 +407,23 @@ static bool patch_steps(felbm_state *s, int64_t n, cudaError_t &err) {
     return true;
 }
 
+// Whether a state on a general mesh with patches takes the patch step: FP32
+// always, and with FP64 coefficients (FP64, FP64 Laplacian) up to one wave of
+// patches, unless the mesh was made for it.  Beyond one wave the patch rows'
+// 18 bytes an entry and the second gradient and mu of the rings cost more than
+// two launches save (jittered Delaunay meshes, us a step, patch step and four
+// launches: FP64 Laplacian 300 x 300 43.1 and 31.2, 600 x 600 153 and 122, 1024
+// x 1024 411 and 347; FP64 223 and 192, 772 and 721, 2101 and 2028).
+static bool patch_wanted(const felbm_state *s) {
+    const felbm_mesh *m = s->mesh;
+    return m->patch_step && ((m->flags & FELBM_MESH_PATCH_STEP) || (s->esize == 4 && !lap_fp64(s)) ||
+                             m->n_nodes <= kOneWave);
+}
+
 template <typename T>
 static int do_steps(felbm_state *s, int64_t n) {
     const felbm_mesh *m = s->mesh;
-    if (m->kind == 0 && m->patch_step) {
+    if (m->kind == 0 && patch_wanted(s)) {
         cudaError_t err = cudaSuccess;
         bool done;
         if constexpr (sizeof(T) == 4)
