@@ -372,8 +372,7 @@ template <typename T, bool LAP64>
 static bool patch_steps(felbm_state *s, int64_t n, cudaError_t &err) {
     const felbm_mesh *m = s->mesh;
     const HostCSR &H = m->host;
-    using CT = typename std::conditional<LAP64, double, T>::type;
-    const size_t smem = patch_smem<T, CT>(H.r1max, H.r2max, H.r3max, H.pemax, H.psmax);
+    const size_t smem = patch_smem<T>(H.r1max, H.r2max, H.r3max, H.pemax, H.psmax);
     if (smem > 227 * 1024) return false;
     const auto kernel = m->n_nodes <= kOneWave ? k_patch_step<T, LAP64, true> : k_patch_step<T, LAP64, false>;
     err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -389,7 +388,8 @@ static bool patch_steps(felbm_state *s, int64_t n, cudaError_t &err) {
     A.pslice = m->d_pslice;
     A.psbase = m->d_psbase;
     A.pcol = m->d_pcol;
-    A.pa = m->d_pa[sizeof(CT) == 8];
+    A.pa = reinterpret_cast<const V2<T> *>(m->d_pa[sizeof(T) == 8]);
+    A.pa64 = reinterpret_cast<const V2<double> *>(m->d_pa[1]);
     A.r1max = H.r1max;
     A.r2max = H.r2max;
     A.r3max = H.r3max;

@@ -37,16 +37,16 @@ struct PatchArgs {
     const int32_t *pslice;  // first slice of each patch in psbase
     const int32_t *psbase;  // first row of 32 entries of each slice
     const uint16_t *pcol;   // region index of each entry
-    const void *pa;         // recovery coefficients of each entry (a_x, a_y; FP64 with LAP64)
+    const V2<T> *pa;        // recovery coefficients of each entry (a_x, a_y)
+    const V2<double> *pa64; // the same in FP64 (LAP64 only)
     int32_t r1max, r2max, r3max, pemax, psmax;
     double kappa64;
 };
 
-// Shared-memory bytes of one block (layout of k_patch_step); C: type of the
-// recovery coefficients.
-template <typename T, typename C>
+// Shared-memory bytes of one block (layout of k_patch_step).
+template <typename T>
 inline size_t patch_smem(int32_t r1max, int32_t r2max, int32_t r3max, int32_t pemax, int32_t psmax) {
-    return (size_t)pemax * 32 * (sizeof(V2<C>) + sizeof(uint16_t)) + (size_t)r2max * sizeof(V2<T>) +
+    return (size_t)pemax * 32 * (sizeof(V2<T>) + sizeof(uint16_t)) + (size_t)r2max * sizeof(V2<T>) +
            (size_t)(r3max + r1max) * sizeof(T) + (size_t)(psmax + 1) * sizeof(int32_t);
 }
 
@@ -56,21 +56,24 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
                  : "memory");
 }
 
-// LAP64: the kappa lap rho term of mu in FP64, as k_mu_lap64 forms it.
+// LAP64: the kappa lap rho term of mu in FP64, as k_mu_lap64 forms it.  Its
+// FP64 coefficients are read from global memory where they are used; staged in
+// place of the FP32 ones, they made every stage convert (the conversions take
+// the FP64 pipe).
 // ONE: all blocks are resident at once with two per SM, whose registers then
 // hold more gathers in flight (jittered Delaunay meshes, FP32, both launches:
 // 256 x 256 10.7 us a step with two blocks per SM, 13.2 with three; 300 x 300,
 // 352 blocks, 17.6 and 13.9; 1024 x 1024 182 and 159).
 template <typename T, bool LAP64, bool ONE>
 __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_patch_step(const __grid_constant__ PatchArgs<T> A) {
-    using CT = typename std::conditional<LAP64, double, T>::type;
+    using CT = typename std::conditional<LAP64, double, T>::type;  // of lap rho
     extern __shared__ __align__(16) unsigned char psm[];
     const DevELL<T> &m = A.c.m;
     const int p = blockIdx.x, tid = threadIdx.x;
     const int32_t n = m.n;
     // (the two cp.async destinations first: whole 32-entry rows keep both, and
     // what follows, 16-byte aligned)
-    V2<CT> *pa = reinterpret_cast<V2<CT> *>(psm);                             // [pemax * 32]
+    V2<T> *pa = reinterpret_cast<V2<T> *>(psm);                               // [pemax * 32]
     uint16_t *pc = reinterpret_cast<uint16_t *>(pa + (size_t)A.pemax * 32);   // [pemax * 32]
     V2<T> *grd = reinterpret_cast<V2<T> *>(pc + (size_t)A.pemax * 32);        // [r2max]
     T *rho = reinterpret_cast<T *>(grd + A.r2max);                            // [r3max]
@@ -80,13 +83,13 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
     const int32_t base = __ldg(A.nbase + p);
     const int4 cnt = __ldg(reinterpret_cast<const int4 *>(A.count) + p);
     const int32_t n0 = cnt.x, n1 = cnt.y, n2 = cnt.z, n3 = cnt.w;
+    const int32_t s0 = __ldg(A.pslice + p), e0 = __ldg(A.psbase + s0);
     {
-        const int32_t s0 = __ldg(A.pslice + p), ns = (n2 + 31) / 32;
-        const int32_t e0 = __ldg(A.psbase + s0), rows = __ldg(A.psbase + s0 + ns) - e0;
+        const int32_t ns = (n2 + 31) / 32, rows = __ldg(A.psbase + s0 + ns) - e0;
         for (int s = tid; s <= ns; s += kPatch) sb[s] = (__ldg(A.psbase + s0 + s) - e0) * 32;
-        const char *ga = reinterpret_cast<const char *>(reinterpret_cast<const V2<CT> *>(A.pa) + (size_t)e0 * 32);
+        const char *ga = reinterpret_cast<const char *>(A.pa + (size_t)e0 * 32);
         const char *gc = reinterpret_cast<const char *>(A.pcol + (size_t)e0 * 32);
-        const int ba = rows * 32 * (int)sizeof(V2<CT>), bc = rows * 64;
+        const int ba = rows * 32 * (int)sizeof(V2<T>), bc = rows * 64;
         for (int b = tid * 16; b < ba; b += kPatch * 16) cp_async16(reinterpret_cast<char *>(pa) + b, ga + b);
         for (int b = tid * 16; b < bc; b += kPatch * 16) cp_async16(reinterpret_cast<char *>(pc) + b, gc + b);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
@@ -107,13 +110,13 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
     __syncthreads();
     V2<T> gs[4];
     {
-        const int e0 = own ? sb[tid >> 5] + (tid & 31) : 0;
+        const int o0 = own ? sb[tid >> 5] + (tid & 31) : 0;
         stream_pairs<T>(m, A.c.fin + 9 * np, np, g, A.c.P.dt, gs, [&](auto &&fn) {
             m.template each_get<false>(row, fn, [&](int k, Ell2<T>) {
                 Ell2<T> v{T(0), T(0)};
                 if (k < row.deg) {
-                    const V2<CT> a = pa[e0 + 32 * k];
-                    v = {(T)a.x, (T)a.y};
+                    const V2<T> a = pa[o0 + 32 * k];
+                    v = {a.x, a.y};
                 }
                 return v;
             });
@@ -128,41 +131,49 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
         rho[r] = chk_idx(j, n, 1u) ? grho[j] : T(0);
     }
     __syncthreads();
-    // fn(j, a) for the entries of region row r (lim: rows in the next ring)
+    // fn(j, a, e) for the entries e of region row r (lim: rows in the next ring)
     auto each = [&](int32_t r, int32_t lim, auto &&fn) {
         const int32_t e1 = sb[(r >> 5) + 1];
 #pragma unroll 4
         for (int32_t e = sb[r >> 5] + (r & 31); e < e1; e += 32) {
             const int j = pc[e];
-            if (chk_idx(j, lim, 2u)) fn(j, pa[e]);
+            if (chk_idx(j, lim, 2u)) fn(j, pa[e], e);
         }
     };
     // 1. recovered grad rho on rings <= 2 (k_grad)
     for (int32_t r = tid; r < n2; r += kPatch) {
         const T fi = rho[r];
         T gx = T(0), gy = T(0);
-        each(r, n3, [&](int j, V2<CT> a) { grad_edge<T>((T)a.x, (T)a.y, rho[j] - fi, gx, gy); });
+        each(r, n3, [&](int j, V2<T> a, int) { grad_edge<T>(a.x, a.y, rho[j] - fi, gx, gy); });
         grd[r] = vset(gx, gy);
     }
     __syncthreads();
     // 2. lap rho and mu on rings <= 1, the stress force at the own node (k_mu)
     T kx_own = T(0), ky_own = T(0);
+    auto lap_of = [&](V2<T> a, int e, V2<T> gi, V2<T> gj, CT &lap) {
+        if constexpr (LAP64) {
+            const double2 c = __ldg(reinterpret_cast<const double2 *>(A.pa64) + (size_t)e0 * 32 + e);
+            lap_edge<CT>(c.x, c.y, gi.x, gi.y, gj.x, gj.y, lap);
+        } else {
+            lap_edge<T>(a.x, a.y, gi.x, gi.y, gj.x, gj.y, lap);
+        }
+    };
     for (int32_t r = tid; r < n1; r += kPatch) {
         const V2<T> gi = grd[r];
         T kx = T(0), ky = T(0);
         CT lap = CT(0);
         if (r < n0) {
-            each(r, n2, [&](int j, V2<CT> a) {
+            each(r, n2, [&](int j, V2<T> a, int e) {
                 const V2<T> gj = grd[j];
-                lap_edge<CT>(a.x, a.y, gi.x, gi.y, gj.x, gj.y, lap);
-                stress_edge<T>((T)a.x, (T)a.y, gi.x, gi.y, gj.x, gj.y, kx, ky);
+                lap_of(a, e, gi, gj, lap);
+                stress_edge<T>(a.x, a.y, gi.x, gi.y, gj.x, gj.y, kx, ky);
             });
             kx_own = A.c.P.kappa * kx;
             ky_own = A.c.P.kappa * ky;
         } else {
-            each(r, n2, [&](int j, V2<CT> a) {
+            each(r, n2, [&](int j, V2<T> a, int e) {
                 const V2<T> gj = grd[j];
-                lap_edge<CT>(a.x, a.y, gi.x, gi.y, gj.x, gj.y, lap);
+                lap_of(a, e, gi, gj, lap);
             });
         }
         if (LAP64)
@@ -176,7 +187,7 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
     T dmx = T(0), dmy = T(0);
     {
         const T fi = mu[tid];
-        each(tid, n1, [&](int j, V2<CT> a) { grad_edge<T>((T)a.x, (T)a.y, mu[j] - fi, dmx, dmy); });
+        each(tid, n1, [&](int j, V2<T> a, int) { grad_edge<T>(a.x, a.y, mu[j] - fi, dmx, dmy); });
     }
     const V2<T> gr = grd[tid];
     collide_write<T>(A.c, g, np, g0, gs, rho_own, gr.x, gr.y, dmx, dmy, kx_own, ky_own);
