@@ -374,7 +374,9 @@ static bool patch_steps(felbm_state *s, int64_t n, cudaError_t &err) {
     const HostCSR &H = m->host;
     const size_t smem = patch_smem<T>(H.r1max, H.r2max, H.r3max, H.pemax, H.psmax);
     if (smem > 227 * 1024) return false;
-    const auto kernel = m->n_nodes <= kOneWave ? k_patch_step<T, LAP64, true> : k_patch_step<T, LAP64, false>;
+    const bool one = m->n_nodes <= kOneWave, lng = m->d_ptail;
+    const auto kernel = one ? (lng ? k_patch_step<T, LAP64, true, true> : k_patch_step<T, LAP64, true, false>)
+                            : (lng ? k_patch_step<T, LAP64, false, true> : k_patch_step<T, LAP64, false, false>);
     err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) {
         cudaGetLastError();
@@ -388,6 +390,8 @@ static bool patch_steps(felbm_state *s, int64_t n, cudaError_t &err) {
     A.pslice = m->d_pslice;
     A.psbase = m->d_psbase;
     A.pcol = m->d_pcol;
+    A.pstail = m->d_pstail;
+    A.ptail = reinterpret_cast<const int2 *>(m->d_ptail);
     A.pa = reinterpret_cast<const V2<T> *>(m->d_pa[sizeof(T) == 8]);
     A.pa64 = reinterpret_cast<const V2<double> *>(m->d_pa[1]);
     A.r1max = H.r1max;
@@ -506,6 +510,8 @@ void mesh_free(felbm_mesh *m) {
     cudaFree(m->d_pnode);
     cudaFree(m->d_pslice);
     cudaFree(m->d_psbase);
+    cudaFree(m->d_pstail);
+    cudaFree(m->d_ptail);
     cudaFree(m->d_pcol);
     for (void *q : m->d_pa) cudaFree(q);
     delete m;
@@ -682,6 +688,10 @@ int felbm_mesh_create(const double *xy, int64_t n_nodes, const int32_t *tri, int
                 up(&m->d_pslice, H.pslice.data(), H.pslice.size() * sizeof(int32_t));
                 up(&m->d_psbase, H.psbase.data(), H.psbase.size() * sizeof(int32_t));
                 up(&m->d_pcol, H.pcol.data(), H.pcol.size() * sizeof(uint16_t));
+                if (!H.ptail.empty()) {
+                    up(&m->d_pstail, H.pstail.data(), H.pstail.size() * sizeof(int32_t));
+                    up(&m->d_ptail, H.ptail.data(), H.ptail.size() * sizeof(int32_t));
+                }
                 const size_t ne = H.pcsr.size();
                 std::vector<float> a32(2 * ne, 0.0f);
                 std::vector<double> a64(2 * ne, 0.0);

@@ -146,17 +146,24 @@ struct HostCSR {
     // [p kPatch, min(n, (p + 1) kPatch))).  Per patch its region: its own
     // nodes, then the nodes 1, 2 and 3 edges away, as internal ids in
     // pnode[pnbase[p] ..); pcount[4 p ..] the counts of rings <= 0, 1, 2, 3.
-    // The rows of rings <= 2 lie in slices of 32 (as DevELL's): pslice[p]
-    // is the patch's first entry of psbase, which holds its slices' first
-    // rows of 32 entries (one more than it has slices); pcol has the region
-    // index and pcsr the CSR entry of each (-1: padding, index of the row).
-    std::vector<int32_t> pnbase, pcount, pnode, pslice, psbase, pcsr;
+    // The rows of rings <= 2 lie in slices of 32 (as DevELL's), with up to
+    // kPatchRow entries of a row; the rest of longer rows follows behind the
+    // patch's slices, row by row, padded to a multiple of 32 (a slice as wide
+    // as its longest row would be 32 times that row).  pslice[p] is the
+    // patch's first entry of psbase, which holds its slices' first rows of 32
+    // entries, their end and the patch's; pcol has the region index and pcsr
+    // the CSR entry of each (-1: padding, index of the row).  pstail (as
+    // psbase) is -1 or the number t of a slice with longer rows, whose row l
+    // has its further entries at [ptail[64 t + 2 l], + ptail[64 t + 2 l + 1])
+    // from the patch's first; both are empty where no row is longer.
+    std::vector<int32_t> pnbase, pcount, pnode, pslice, psbase, pcsr, pstail, ptail;
     std::vector<uint16_t> pcol;
     int32_t r1max = 0, r2max = 0, r3max = 0;  // largest ring <= 1, 2, 3 sizes
     int32_t pemax = 0, psmax = 0;             // most rows of 32 entries, most slices of a patch
 };
 
-constexpr int kPatch = 256;  // nodes per patch of general triangle meshes
+constexpr int kPatch = 256;   // nodes per patch of general triangle meshes
+constexpr int kPatchRow = 32;  // entries of a row in a patch's slices
 
 // General tetrahedral mesh (3-D), same conventions: for each neighbour j != i
 // a_ij = sum_{T∋i,j} |T| grad N_j / (4 m_i) (3 components) and the symmetric
@@ -522,6 +529,7 @@ struct felbm_mesh {
     // patches of general triangle meshes (HostCSR), with the recovery
     // coefficients a of their rows per precision {FP32, FP64}
     int32_t *d_pnbase = nullptr, *d_pcount = nullptr, *d_pnode = nullptr, *d_pslice = nullptr, *d_psbase = nullptr;
+    int32_t *d_pstail = nullptr, *d_ptail = nullptr;
     uint16_t *d_pcol = nullptr;
     void *d_pa[2] = {nullptr, nullptr};
     bool patch_step = false;

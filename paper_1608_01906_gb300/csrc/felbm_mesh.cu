@@ -217,7 +217,8 @@ static void build_patches(HostCSR &H) {
         const int32_t slices = (cnt[2] + 31) / 32;
         // region indices are 16-bit, entry offsets 32-bit: else no patch step
         if (reg.size() > 65535 || H.pcsr.size() > (size_t)0x60000000) {
-            for (auto *v : {&H.pnbase, &H.pcount, &H.pnode, &H.pslice, &H.psbase, &H.pcsr}) v->clear();
+            for (auto *v : {&H.pnbase, &H.pcount, &H.pnode, &H.pslice, &H.psbase, &H.pcsr, &H.pstail, &H.ptail})
+                v->clear();
             H.pcol.clear();
             return;
         }
@@ -231,6 +232,9 @@ static void build_patches(HostCSR &H) {
             int32_t w = 0;
             for (int32_t r = 32 * s; r < std::min(cnt[2], 32 * (s + 1)); ++r)
                 w = std::max(w, H.rowptr[reg[r] + 1] - H.rowptr[reg[r]]);
+            H.pstail.push_back(w > kPatchRow ? (int32_t)(H.ptail.size() / 64) : -1);
+            if (w > kPatchRow) H.ptail.resize(H.ptail.size() + 64, 0);
+            w = std::min(w, kPatchRow);
             for (int32_t k = 0; k < w; ++k)
                 for (int32_t r = 32 * s; r < 32 * (s + 1); ++r) {
                     const int32_t g = reg[std::min(r, cnt[2] - 1)];
@@ -241,12 +245,27 @@ static void build_patches(HostCSR &H) {
                 }
         }
         H.psbase.push_back((int32_t)(H.pcsr.size() / 32));
+        for (int32_t r = 0; r < cnt[2]; ++r) {
+            const int32_t t = H.pstail[(size_t)H.pslice[p] + r / 32], g = reg[r];
+            const int32_t further = H.rowptr[g + 1] - H.rowptr[g] - kPatchRow;
+            if (t < 0 || further <= 0) continue;
+            H.ptail[(size_t)64 * t + 2 * (r % 32)] = (int32_t)(H.pcsr.size() - 32 * first);
+            H.ptail[(size_t)64 * t + 2 * (r % 32) + 1] = further;
+            for (int32_t e = H.rowptr[g] + kPatchRow; e < H.rowptr[g + 1]; ++e) {
+                H.pcsr.push_back(e);
+                H.pcol.push_back((uint16_t)loc[H.col[e]]);
+            }
+        }
+        for (; H.pcsr.size() % 32; H.pcol.push_back(0)) H.pcsr.push_back(-1);
+        H.psbase.push_back((int32_t)(H.pcsr.size() / 32));
+        H.pstail.insert(H.pstail.end(), 2, -1);
         H.pemax = std::max(H.pemax, (int32_t)(H.pcsr.size() / 32 - first));
         H.psmax = std::max(H.psmax, slices);
         H.r1max = std::max(H.r1max, cnt[1]);
         H.r2max = std::max(H.r2max, cnt[2]);
         H.r3max = std::max(H.r3max, cnt[3]);
     }
+    if (H.ptail.empty()) H.pstail.clear();
 }
 
 // Conformity of a P1 triangulation (the Galerkin streaming of Sec. 2.2.1

@@ -35,7 +35,9 @@ struct PatchArgs {
     const int32_t *count;   // per patch: nodes of rings <= 0, 1, 2, 3
     const int32_t *node;    // region nodes (internal ids), own first
     const int32_t *pslice;  // first slice of each patch in psbase
-    const int32_t *psbase;  // first row of 32 entries of each slice
+    const int32_t *psbase;  // first row of 32 entries of each slice, their end, the patch's end
+    const int32_t *pstail;  // of each slice: -1, or its table of further entries (LONG)
+    const int2 *ptail;      // first of them (from the patch's first entry) and count, 32 a table
     const uint16_t *pcol;   // region index of each entry
     const V2<T> *pa;        // recovery coefficients of each entry (a_x, a_y)
     const V2<double> *pa64; // the same in FP64 (LAP64 only)
@@ -64,7 +66,8 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 // hold more gathers in flight (jittered Delaunay meshes, FP32, both launches:
 // 256 x 256 10.7 us a step with two blocks per SM, 13.2 with three; 300 x 300,
 // 352 blocks, 17.6 and 13.9; 1024 x 1024 182 and 159).
-template <typename T, bool LAP64, bool ONE>
+// LONG: some rows have entries behind the slices (HostCSR::ptail).
+template <typename T, bool LAP64, bool ONE, bool LONG>
 __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_patch_step(const __grid_constant__ PatchArgs<T> A) {
     using CT = typename std::conditional<LAP64, double, T>::type;  // of lap rho
     extern __shared__ __align__(16) unsigned char psm[];
@@ -85,7 +88,7 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
     const int32_t n0 = cnt.x, n1 = cnt.y, n2 = cnt.z, n3 = cnt.w;
     const int32_t s0 = __ldg(A.pslice + p), e0 = __ldg(A.psbase + s0);
     {
-        const int32_t ns = (n2 + 31) / 32, rows = __ldg(A.psbase + s0 + ns) - e0;
+        const int32_t ns = (n2 + 31) / 32, rows = __ldg(A.psbase + s0 + ns + 1) - e0;
         for (int s = tid; s <= ns; s += kPatch) sb[s] = (__ldg(A.psbase + s0 + s) - e0) * 32;
         const char *ga = reinterpret_cast<const char *>(A.pa + (size_t)e0 * 32);
         const char *gc = reinterpret_cast<const char *>(A.pcol + (size_t)e0 * 32);
@@ -109,13 +112,20 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
     V2<T> gs[4];
+    // the entries of region row r behind the slices
+    auto further = [&](int32_t r) {
+        int32_t t = -1;
+        if (LONG) t = __ldg(A.pstail + s0 + (r >> 5));
+        return t < 0 ? make_int2(0, 0) : __ldg(A.ptail + 32 * (size_t)t + (r & 31));
+    };
     {
         const int o0 = own ? sb[tid >> 5] + (tid & 31) : 0;
+        const int2 q0 = further(own ? tid : 0);
         stream_pairs<T>(m, A.c.fin + 9 * np, np, g, A.c.P.dt, gs, [&](auto &&fn) {
             m.template each_get<false>(row, fn, [&](int k, Ell2<T>) {
                 Ell2<T> v{T(0), T(0)};
-                if (k < row.deg) {
-                    const V2<T> a = pa[o0 + 32 * k];
+                if (k < row.deg && (!LONG || k < kPatchRow + q0.y)) {
+                    const V2<T> a = pa[!LONG || k < kPatchRow ? o0 + 32 * k : q0.x + (k - kPatchRow)];
                     v = {a.x, a.y};
                 }
                 return v;
@@ -138,6 +148,14 @@ __global__ void __launch_bounds__(kPatch, sizeof(T) == 4 ? (ONE ? 2 : 3) : 1) k_
         for (int32_t e = sb[r >> 5] + (r & 31); e < e1; e += 32) {
             const int j = pc[e];
             if (chk_idx(j, lim, 2u)) fn(j, pa[e], e);
+        }
+        if (LONG) {
+            const int2 q = further(r);
+#pragma unroll 4
+            for (int32_t e = q.x; e < q.x + q.y; ++e) {
+                const int j = pc[e];
+                if (chk_idx(j, lim, 2u)) fn(j, pa[e], e);
+            }
         }
     };
     // 1. recovered grad rho on rings <= 2 (k_grad)
