@@ -121,8 +121,8 @@ typedef struct felbm_params {
  * order within a patch.  A general mesh steps in two launches per step (the
  * streamed h and rho, then one block per patch with the patch's nodes up to
  * 3 edges away staged in shared memory) or in four over global fields: FP32
- * states take two, those with FP64 coefficients (FP64, FELBM_PARAM_LAP_FP64)
- * two up to 77,824 nodes.  FELBM_MESH_PATCH_STEP and FELBM_MESH_SPLIT_STEP
+ * states take two, FP64 ones two up to 77,824 nodes or with a node of more
+ * than 32 neighbours.  FELBM_MESH_PATCH_STEP and FELBM_MESH_SPLIT_STEP
  * force one of the two (a mesh whose patches do not fit shared memory takes
  * four launches all the same); both give the same results bit for bit.
  * A mesh that is the structured split of a unit lattice

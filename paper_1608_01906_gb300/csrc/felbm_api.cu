@@ -411,17 +411,18 @@ static bool patch_steps(felbm_state *s, int64_t n, cudaError_t &err) {
     return true;
 }
 
-// Whether a state on a general mesh with patches takes the patch step: FP32
-// always, and with FP64 coefficients (FP64, FP64 Laplacian) up to one wave of
-// patches, unless the mesh was made for it.  Beyond one wave the patch rows'
-// 18 bytes an entry and the second gradient and mu of the rings cost more than
-// two launches save (jittered Delaunay meshes, us a step, patch step and four
-// launches: FP64 Laplacian 300 x 300 43.1 and 31.2, 600 x 600 153 and 122, 1024
-// x 1024 411 and 347; FP64 223 and 192, 772 and 721, 2101 and 2028).
+// Whether a state on a general mesh with patches takes the patch step: always
+// in FP32; in FP64, whose arithmetic on the rings costs more than two launches
+// save beyond one wave of patches, up to there, where a row is so long that its
+// one thread bounds a pass, or on a mesh made for it.  Jittered Delaunay meshes,
+// us a step, patch step and four launches: FP64 300 x 300 223 and 192, 600 x 600
+// 772 and 721, 1024 x 1024 2102 and 2030, with a hub of 150 neighbours 600 x 600
+// 901 and 1065; FP64 Laplacian 300 x 300 29.1 and 31.3, 600 x 600 111 and 123,
+// 1024 x 1024 272 and 347.
 static bool patch_wanted(const felbm_state *s) {
     const felbm_mesh *m = s->mesh;
-    return m->patch_step && ((m->flags & FELBM_MESH_PATCH_STEP) || (s->esize == 4 && !lap_fp64(s)) ||
-                             m->n_nodes <= kOneWave);
+    return m->patch_step &&
+           ((m->flags & FELBM_MESH_PATCH_STEP) || s->esize == 4 || m->n_nodes <= kOneWave || m->d_ptail);
 }
 
 template <typename T>

@@ -36,7 +36,7 @@ def run(mesh_args, precision, lap_fp64, **step):
     return got, launches
 
 
-@pytest.mark.parametrize("precision, lap_fp64, default", [("fp32", False, STEPS), ("fp32", True, 0), ("fp64", False, 0)])
+@pytest.mark.parametrize("precision, lap_fp64, default", [("fp32", False, STEPS), ("fp32", True, STEPS), ("fp64", False, 0)])
 def test_patch_and_four_launch_step_bitwise(mesh_args, precision, lap_fp64, default):
     a, na = run(mesh_args, precision, lap_fp64, patch_step=True)
     b, nb = run(mesh_args, precision, lap_fp64, split_step=True)
