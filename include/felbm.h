@@ -173,7 +173,8 @@ int felbm_mesh_create_tet(const double *xyz, int64_t n_nodes, const int32_t *tet
 /* Mesh facts.  Any output pointer may be NULL.  kind: 0 = general
  * (unstructured kernels), 1 = structured lattice, 2 = tetrahedral,
  * 3 = Kuhn tetrahedral lattice (n_tri then counts tetrahedra).  device_bytes: device memory held by the
- * mesh. */
+ * mesh.  A general mesh uploads its rows for the first state that reads them
+ * (each precision its own), so this grows with the first states on it. */
 int felbm_mesh_info(const felbm_mesh *mesh, int64_t *n_nodes, int64_t *n_tri, int32_t *kind,
                     int64_t *device_bytes);
 

@@ -53,14 +53,15 @@ int cuda_status(cudaError_t e) {
         if (_e != cudaSuccess) return cuda_status(_e); \
     } while (0)
 
+// with_b false: for kernels that read no b_xx, b_xy (a stands in for them)
 template <typename T>
-static DevELL<T> dev_ell(const felbm_mesh *m) {
+static DevELL<T> dev_ell(const felbm_mesh *m, bool with_b = true) {
     DevELL<T> d;
     d.n = (int32_t)m->n_nodes;
     d.sbase = m->d_sbase;
     void *const *e = m->d_ell[sizeof(T) == 8];
     d.a = reinterpret_cast<const Ell2<T> *>(e[0]);
-    d.b = reinterpret_cast<const Ell2<T> *>(e[1]);
+    d.b = reinterpret_cast<const Ell2<T> *>(e[with_b ? 1 : 0]);
     d.c = reinterpret_cast<const Ell2<T> *>(e[2]);
     d.deg = m->d_deg;
     d.tag = m->d_tag;
@@ -85,10 +86,29 @@ cudaError_t mesh_upload(felbm_mesh *m, void **d, const void *host, size_t bytes)
     return bytes ? cudaMemcpy(*d, host, bytes, cudaMemcpyHostToDevice) : cudaSuccess;
 }
 
-// The entries of DevELL<T> (slices sb) from the assembled rows.
+cudaError_t mesh_hold(felbm_mesh *m, void **d, const void *host, size_t bytes) {
+    if (*d) return cudaSuccess;
+    void *p = nullptr;
+    cudaError_t e = cudaMalloc(&p, std::max<size_t>(bytes, 1));
+    if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(p, host, bytes, cudaMemcpyHostToDevice, m->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
+    if (e != cudaSuccess) {
+        cudaFree(p);
+        return e;
+    }
+    *d = p;
+    m->device_bytes += (int64_t)bytes;
+    return cudaSuccess;
+}
+
+// The entries of DevELL<T> from the assembled rows, on the device; the b_xx,
+// b_xy among them where wanted.
 template <typename T>
-static cudaError_t upload_ell(felbm_mesh *m, const std::vector<int32_t> &sb) {
+static cudaError_t hold_ell(felbm_mesh *m, bool with_b) {
     const HostCSR &H = m->host;
+    void **d = m->d_ell[sizeof(T) == 8];
+    if (d[0] && d[2] && (d[1] || !with_b)) return cudaSuccess;
+    const std::vector<int32_t> sb = ell_slices(H.n, H.rowptr);
     const size_t entries = (size_t)sb.back() * 32;
     std::vector<Ell2<T>> a(entries), b(entries), c(entries);
     for (size_t s = 0; s + 1 < sb.size(); ++s)
@@ -106,10 +126,9 @@ static cudaError_t upload_ell(felbm_mesh *m, const std::vector<int32_t> &sb) {
                     c[p] = {T(0), ell_id<T>((int32_t)i)};
                 }
             }
-    void **d = m->d_ell[sizeof(T) == 8];
-    cudaError_t e = mesh_upload(m, &d[0], a.data(), entries * sizeof(Ell2<T>));
-    if (e == cudaSuccess) e = mesh_upload(m, &d[1], b.data(), entries * sizeof(Ell2<T>));
-    if (e == cudaSuccess) e = mesh_upload(m, &d[2], c.data(), entries * sizeof(Ell2<T>));
+    cudaError_t e = mesh_hold(m, &d[0], a.data(), entries * sizeof(Ell2<T>));
+    if (e == cudaSuccess && with_b) e = mesh_hold(m, &d[1], b.data(), entries * sizeof(Ell2<T>));
+    if (e == cudaSuccess) e = mesh_hold(m, &d[2], c.data(), entries * sizeof(Ell2<T>));
     return e;
 }
 
@@ -208,7 +227,7 @@ static double kappa64(const felbm_params &p) {
 static bool lap_fp64(const felbm_state *s) { return s->esize == 4 && (s->params.flags & FELBM_PARAM_LAP_FP64); }
 
 // The mesh's operators with FP64 coefficients, for the FP64 Laplacian.
-static DevELL<double> topo64(const felbm_mesh *m, const DevELL<float> &) { return dev_ell<double>(m); }
+static DevELL<double> topo64(const felbm_mesh *m, const DevELL<float> &) { return dev_ell<double>(m, false); }
 static DevLattice<double> topo64(const felbm_mesh *m, const DevLattice<float> &) { return dev_lattice<double>(m); }
 
 template <typename T, typename Topo>
@@ -365,22 +384,26 @@ static cudaError_t lat_smem_attr() {
     return cudaSuccess;
 }
 
-// Two launches per step over a general triangle mesh with patches; false
-// when the patch kernel's shared memory exceeds what a block can have (the
-// four-launch step then runs).
+// Shared memory of the patch kernel on a mesh.
+template <typename T>
+static size_t patch_bytes(const felbm_mesh *m) {
+    const HostCSR &H = m->host;
+    return patch_smem<T>(H.r1max, H.r2max, H.r3max, H.pemax, H.psmax);
+}
+
+// Two launches per step over a general triangle mesh with patches.
 template <typename T, bool LAP64>
-static bool patch_steps(felbm_state *s, int64_t n, cudaError_t &err) {
+static cudaError_t patch_steps(felbm_state *s, int64_t n) {
     const felbm_mesh *m = s->mesh;
     const HostCSR &H = m->host;
-    const size_t smem = patch_smem<T>(H.r1max, H.r2max, H.r3max, H.pemax, H.psmax);
-    if (smem > 227 * 1024) return false;
-    const bool one = m->n_nodes <= kOneWave, lng = m->d_ptail;
+    const size_t smem = patch_bytes<T>(m);
+    const bool one = m->n_nodes <= kOneWave, lng = !H.ptail.empty();
     const auto kernel = one ? (lng ? k_patch_step<T, LAP64, true, true> : k_patch_step<T, LAP64, true, false>)
                             : (lng ? k_patch_step<T, LAP64, false, true> : k_patch_step<T, LAP64, false, false>);
-    err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) {
         cudaGetLastError();
-        return true;
+        return err;
     }
     const DevELL<T> d = dev_ell<T>(m);
     PatchArgs<T> A;
@@ -408,11 +431,11 @@ static bool patch_steps(felbm_state *s, int64_t n, cudaError_t &err) {
         prof_end(s, sl);
         s->cur ^= 1;
     }
-    return true;
+    return cudaSuccess;
 }
 
-// Whether a state on a general mesh with patches takes the patch step: always
-// in FP32; in FP64, whose arithmetic on the rings costs more than two launches
+// Whether a state on a general mesh takes the patch step: where the mesh has
+// patches and a block their shared memory, always in FP32; in FP64, whose arithmetic on the rings costs more than two launches
 // save beyond one wave of patches, up to there, where a row is so long that its
 // one thread bounds a pass, or on a mesh made for it.  Jittered Delaunay meshes,
 // us a step, patch step and four launches: FP64 300 x 300 223 and 192, 600 x 600
@@ -421,21 +444,56 @@ static bool patch_steps(felbm_state *s, int64_t n, cudaError_t &err) {
 // 1024 x 1024 272 and 347.
 static bool patch_wanted(const felbm_state *s) {
     const felbm_mesh *m = s->mesh;
-    return m->patch_step &&
-           ((m->flags & FELBM_MESH_PATCH_STEP) || s->esize == 4 || m->n_nodes <= kOneWave || m->d_ptail);
+    if (m->kind != 0 || !m->patch_step ||
+        (s->esize == 8 ? patch_bytes<double>(m) : patch_bytes<float>(m)) > 227 * 1024)
+        return false;
+    return (m->flags & FELBM_MESH_PATCH_STEP) || s->esize == 4 || m->n_nodes <= kOneWave || !m->host.ptail.empty();
+}
+
+// The device arrays of a general mesh that state s reads: its precision's
+// rows, with the FP64 Laplacian the FP64 a_ij and neighbours too, and the
+// patches if it takes the patch step.
+static cudaError_t hold_rows(felbm_mesh *m, const felbm_state *s) {
+    const HostCSR &H = m->host;
+    const bool f32 = s->esize == 4, lap = lap_fp64(s);
+    const std::lock_guard<std::mutex> guard(m->lock);
+    cudaError_t e = f32 ? hold_ell<float>(m, true) : cudaSuccess;
+    if (e == cudaSuccess && (!f32 || lap)) e = hold_ell<double>(m, !f32);
+    if (e != cudaSuccess || !patch_wanted(s)) return e;
+    auto hold = [&](auto *&d, const auto &v) {
+        if (e == cudaSuccess && !v.empty()) e = mesh_hold(m, (void **)&d, v.data(), v.size() * sizeof(v[0]));
+    };
+    hold(m->d_pnbase, H.pnbase);
+    hold(m->d_pcount, H.pcount);
+    hold(m->d_pnode, H.pnode);
+    hold(m->d_pslice, H.pslice);
+    hold(m->d_psbase, H.psbase);
+    hold(m->d_pstail, H.pstail);
+    hold(m->d_ptail, H.ptail);
+    hold(m->d_pcol, H.pcol);
+    auto hold_a = [&](void *&d, auto zero) {
+        if (e != cudaSuccess || d) return;
+        std::vector<decltype(zero)> a(2 * H.pcsr.size(), zero);
+        for (size_t k = 0; k < H.pcsr.size(); ++k)
+            if (H.pcsr[k] >= 0) {
+                a[2 * k] = (decltype(zero))H.ax[H.pcsr[k]];
+                a[2 * k + 1] = (decltype(zero))H.ay[H.pcsr[k]];
+            }
+        hold(d, a);
+    };
+    if (f32) hold_a(m->d_pa[0], 0.0f);
+    if (!f32 || lap) hold_a(m->d_pa[1], 0.0);
+    return e;
 }
 
 template <typename T>
 static int do_steps(felbm_state *s, int64_t n) {
     const felbm_mesh *m = s->mesh;
-    if (m->kind == 0 && patch_wanted(s)) {
-        cudaError_t err = cudaSuccess;
-        bool done;
-        if constexpr (sizeof(T) == 4)
-            done = lap_fp64(s) ? patch_steps<T, true>(s, n, err) : patch_steps<T, false>(s, n, err);
-        else
-            done = patch_steps<T, false>(s, n, err);
-        if (done) return cuda_status(err);
+    if (patch_wanted(s)) {
+        if constexpr (sizeof(T) == 4) {
+            if (lap_fp64(s)) return cuda_status(patch_steps<T, true>(s, n));
+        }
+        return cuda_status(patch_steps<T, false>(s, n));
     }
     if (m->kind == 1) {
         const bool l64 = lap_fp64(s);
@@ -680,30 +738,6 @@ int felbm_mesh_create(const double *xy, int64_t n_nodes, const int32_t *tri, int
             for (size_t k = 0; k < N; ++k) deg[k] = (uint8_t)std::min(255, H.rowptr[k + 1] - H.rowptr[k]);
             up(&m->d_sbase, sb.data(), sb.size() * sizeof(int32_t));
             up(&m->d_deg, deg.data(), N);
-            if (e == cudaSuccess) e = upload_ell<float>(m, sb);
-            if (e == cudaSuccess) e = upload_ell<double>(m, sb);
-            if (m->patch_step) {
-                up(&m->d_pnbase, H.pnbase.data(), H.pnbase.size() * sizeof(int32_t));
-                up(&m->d_pcount, H.pcount.data(), H.pcount.size() * sizeof(int32_t));
-                up(&m->d_pnode, H.pnode.data(), H.pnode.size() * sizeof(int32_t));
-                up(&m->d_pslice, H.pslice.data(), H.pslice.size() * sizeof(int32_t));
-                up(&m->d_psbase, H.psbase.data(), H.psbase.size() * sizeof(int32_t));
-                up(&m->d_pcol, H.pcol.data(), H.pcol.size() * sizeof(uint16_t));
-                if (!H.ptail.empty()) {
-                    up(&m->d_pstail, H.pstail.data(), H.pstail.size() * sizeof(int32_t));
-                    up(&m->d_ptail, H.ptail.data(), H.ptail.size() * sizeof(int32_t));
-                }
-                const size_t ne = H.pcsr.size();
-                std::vector<float> a32(2 * ne, 0.0f);
-                std::vector<double> a64(2 * ne, 0.0);
-                for (size_t k = 0; k < ne; ++k)
-                    if (H.pcsr[k] >= 0) {
-                        a32[2 * k] = (float)(a64[2 * k] = H.ax[H.pcsr[k]]);
-                        a32[2 * k + 1] = (float)(a64[2 * k + 1] = H.ay[H.pcsr[k]]);
-                    }
-                up(&m->d_pa[0], a32.data(), 2 * ne * sizeof(float));
-                up(&m->d_pa[1], a64.data(), 2 * ne * sizeof(double));
-            }
         } catch (const std::bad_alloc &) {
             e = cudaErrorMemoryAllocation;
         }
@@ -723,7 +757,10 @@ int felbm_mesh_info(const felbm_mesh *m, int64_t *n_nodes, int64_t *n_tri, int32
     if (n_nodes) *n_nodes = m->n_nodes;
     if (n_tri) *n_tri = m->n_tri;
     if (kind) *kind = m->kind;
-    if (device_bytes) *device_bytes = m->device_bytes;
+    if (device_bytes) {
+        const std::lock_guard<std::mutex> guard(m->lock);
+        *device_bytes = m->device_bytes;
+    }
     return FELBM_OK;
 }
 
@@ -757,6 +794,13 @@ int felbm_state_init(const felbm_mesh *mesh, const felbm_params *params, const d
     alloc(&s->mom, 4 * N * es);
     alloc((void **)&s->d_out, (5 * N + 3 * (kTotalsBlocks + 1)) * sizeof(double));
     alloc((void **)&s->d_flag, sizeof(int));
+    if (e == cudaSuccess && mesh->kind == 0) {
+        try {
+            e = hold_rows(const_cast<felbm_mesh *>(mesh), s);
+        } catch (const std::bad_alloc &) {
+            e = cudaErrorMemoryAllocation;
+        }
+    }
     if (e != cudaSuccess) {
         int rs = cuda_status(e);
         state_free(s);

@@ -39,10 +39,14 @@ static DevELL3<T> dev_ell3(const felbm_mesh *m) {
     return d;
 }
 
-// The entries of DevELL3<T> (slices sb) from the assembled rows.
+// The entries of DevELL3<T> from the assembled rows, on the device.
 template <typename T>
-static cudaError_t upload_ell3(felbm_mesh *m, const std::vector<int32_t> &sb) {
+static cudaError_t hold_ell3(felbm_mesh *m) {
     const HostCSR3 &H = m->host3;
+    void **d = m->d_ell[sizeof(T) == 8];
+    const std::lock_guard<std::mutex> guard(m->lock);
+    if (d[0] && d[1] && d[2]) return cudaSuccess;
+    const std::vector<int32_t> sb = ell_slices(H.n, H.rowptr);
     const size_t entries = (size_t)sb.back() * 32, nnz = H.col.size();
     const double *cf = H.coef.data();
     std::vector<Ell4<T>> a(entries), b(entries);
@@ -63,10 +67,9 @@ static cudaError_t upload_ell3(felbm_mesh *m, const std::vector<int32_t> &sb) {
                     b[p] = {T(0), T(0), T(0), T(0)};
                 }
             }
-    void **d = m->d_ell[sizeof(T) == 8];
-    cudaError_t e = mesh_upload(m, &d[0], a.data(), entries * sizeof(Ell4<T>));
-    if (e == cudaSuccess) e = mesh_upload(m, &d[1], b.data(), entries * sizeof(Ell4<T>));
-    if (e == cudaSuccess) e = mesh_upload(m, &d[2], c.data(), 2 * entries * sizeof(T));
+    cudaError_t e = mesh_hold(m, &d[0], a.data(), entries * sizeof(Ell4<T>));
+    if (e == cudaSuccess) e = mesh_hold(m, &d[1], b.data(), entries * sizeof(Ell4<T>));
+    if (e == cudaSuccess) e = mesh_hold(m, &d[2], c.data(), 2 * entries * sizeof(T));
     return e;
 }
 
@@ -297,6 +300,14 @@ int state_init3(const felbm_mesh *mesh, const felbm_params *params, const double
     alloc(&s->mom, 5 * N * es);
     alloc((void **)&s->d_out, (6 * N + 4 * (kTotalsBlocks + 1)) * sizeof(double));
     alloc((void **)&s->d_flag, sizeof(int));
+    if (e == cudaSuccess && mesh->kind == 2) {
+        felbm_mesh *m = const_cast<felbm_mesh *>(mesh);
+        try {
+            e = es == 8 ? hold_ell3<double>(m) : hold_ell3<float>(m);
+        } catch (const std::bad_alloc &) {
+            e = cudaErrorMemoryAllocation;
+        }
+    }
     if (e != cudaSuccess) {
         const int rs = cuda_status(e);
         state_free(s);
@@ -481,8 +492,6 @@ extern "C" int felbm_mesh_create_tet(const double *xyz, int64_t n_nodes, const i
             const std::vector<int32_t> sb = ell_slices(H.n, H.rowptr);
             if (e == cudaSuccess)
                 e = mesh_upload(m, (void **)&m->d_sbase, sb.data(), sb.size() * sizeof(int32_t));
-            if (e == cudaSuccess) e = upload_ell3<float>(m, sb);
-            if (e == cudaSuccess) e = upload_ell3<double>(m, sb);
         } catch (const std::bad_alloc &) {
             e = cudaErrorMemoryAllocation;
         }

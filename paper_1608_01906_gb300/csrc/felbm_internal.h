@@ -5,6 +5,7 @@
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <utility>
 #include <vector>
 
@@ -520,7 +521,9 @@ struct felbm_mesh {
     // device arrays
     int32_t *d_perm = nullptr;
     // general meshes (kinds 0 and 2): rows in slices of 32 nodes, per
-    // precision {FP32, FP64} the entries of DevELL / DevELL3
+    // precision {FP32, FP64} the entries of DevELL / DevELL3.  These and the
+    // patches' arrays are uploaded for the first state that reads them
+    // (mesh_hold) and stay as long as the mesh.
     int32_t *d_sbase = nullptr;
     void *d_ell[2][4] = {};
     uint8_t *d_deg = nullptr;  // neighbours of each node (kind 0)
@@ -533,6 +536,7 @@ struct felbm_mesh {
     uint16_t *d_pcol = nullptr;
     void *d_pa[2] = {nullptr, nullptr};
     bool patch_step = false;
+    mutable std::mutex lock;  // of the uploads for new states and device_bytes
     int64_t device_bytes = 0;
 };
 
@@ -584,6 +588,10 @@ int cuda_status(cudaError_t e);
 // Upload `bytes` of host data to a new device array of mesh m (counted in
 // its device_bytes).
 cudaError_t mesh_upload(felbm_mesh *m, void **d, const void *host, size_t bytes);
+// Upload `bytes` of host data to the device array *d of mesh m unless it is
+// there already, on the mesh's stream and waiting for it (as state creation
+// does); *d stays null where that fails.  Under m's lock.
+cudaError_t mesh_hold(felbm_mesh *m, void **d, const void *host, size_t bytes);
 // Slices of 32 rows: sbase[s] is the first of slice s's rows of 32 entries,
 // as many as the longest of its CSR rows.
 std::vector<int32_t> ell_slices(int32_t n, const std::vector<int32_t> &rowptr);

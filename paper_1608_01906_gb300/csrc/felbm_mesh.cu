@@ -215,8 +215,10 @@ static void build_patches(HostCSR &H) {
             cnt[ring] = (int32_t)reg.size();
         }
         const int32_t slices = (cnt[2] + 31) / 32;
-        // region indices are 16-bit, entry offsets 32-bit: else no patch step
-        if (reg.size() > 65535 || H.pcsr.size() > (size_t)0x60000000) {
+        // region indices are 16-bit, entry offsets 32-bit, and a block has 227 KB
+        // of shared memory for the region's fields (FP32 grad rho, rho and mu of
+        // rings <= 2, 3 and 1): else no patch step
+        if (reg.size() > 65535 || 8 * (size_t)cnt[2] + 4 * ((size_t)cnt[3] + cnt[1]) > 227 * 1024 || H.pcsr.size() > (size_t)0x60000000) {
             for (auto *v : {&H.pnbase, &H.pcount, &H.pnode, &H.pslice, &H.psbase, &H.pcsr, &H.pstail, &H.ptail})
                 v->clear();
             H.pcol.clear();
