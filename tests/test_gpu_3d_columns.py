@@ -45,3 +45,19 @@ def test_fp32_two_node_columns(size, walls):
     a, b = (run(args, prm, precision, 10, 3) for precision in ("fp32", "fp64"))
     assert rel_l2(a["rho"], b["rho"]) <= 2e-6, rel_l2(a["rho"], b["rho"])
     assert rel_l2(a["u"], b["u"]) <= 1e-5, rel_l2(a["u"], b["u"])
+
+
+# (planes that are no multiple of a block, and an odd height: the last column
+# of a periodic lattice has one node, the first and last of a walled one mix a
+# wall layer with an inner one)
+@pytest.mark.parametrize("walls", [False, True])
+def test_fp32_two_node_columns_odd_height(walls):
+    args, prm = lattice((67, 61, 65), walls)
+    a, b = (run(args, prm, precision, 10, 3) for precision in ("fp32", "fp64"))
+    assert rel_l2(a["rho"], b["rho"]) <= 2e-6, rel_l2(a["rho"], b["rho"])
+    assert rel_l2(a["u"], b["u"]) <= 1e-5, rel_l2(a["u"], b["u"])
+
+
+@pytest.mark.parametrize("walls", [False, True])
+def test_fp64_thread_per_node(walls):
+    check_oracle(*lattice((43, 41, 39), walls), 3, 3)  # 68,757 nodes
