@@ -84,7 +84,7 @@ __device__ __forceinline__ const LatCoef<T> &batch_coef(const BatchArgs<T> &B, c
 }
 
 template <typename T, bool SC>
-__global__ void __launch_bounds__(kNT, (sizeof(T) == 4 ? 768 : 512) / kNT) k_batch_step(const __grid_constant__ BatchArgs<T> B) {
+__global__ void __launch_bounds__(kNT, 768 / kNT) k_batch_step(const __grid_constant__ BatchArgs<T> B) {
     __shared__ StepSmem<T> S;
     __shared__ __align__(16) LatArgs<T> sA;
     extern __shared__ __align__(128) unsigned char bdsm[];
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kNT, (sizeof(T) == 4 ? 768 : 512) / kNT) k_bat
 // the single-mesh step (4 blocks per SM in FP32).  Zeroes both tile counters,
 // so that a walking launch after it starts from zero.
 template <typename T, bool SC>
-__global__ void __launch_bounds__(kNT, (sizeof(T) == 4 ? 1024 : 512) / kNT) k_batch_tile(const __grid_constant__ BatchArgs<T> B) {
+__global__ void __launch_bounds__(kNT, 1024 / kNT) k_batch_tile(const __grid_constant__ BatchArgs<T> B) {
     __shared__ StepSmem<T> S;
     __shared__ __align__(16) LatArgs<T> sA;
     extern __shared__ __align__(128) unsigned char bdsm[];

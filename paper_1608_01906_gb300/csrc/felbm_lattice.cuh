@@ -1024,7 +1024,7 @@ __device__ __forceinline__ bool take_next(const StepSmem<T> &S, TilePipe &pp) {
 // node, no better issue rate), so that walk is left to the batched kernel.
 // LAP64: the kappa lap rho term of mu in FP64 (FELBM_PARAM_LAP_FP64).
 template <typename T, bool LAP64 = false>
-__global__ void __launch_bounds__(kNT, (sizeof(T) == 4 ? 1024 : 512) / kNT) k_lat_step(LatArgs<T> A) {
+__global__ void __launch_bounds__(kNT, 1024 / kNT) k_lat_step(LatArgs<T> A) {
     __shared__ StepSmem<T> S;
     extern __shared__ __align__(128) unsigned char lat_dsm[];
     lat_block_init<T>(S);

@@ -57,8 +57,8 @@ static bool encode(PFN_cuTensorMapEncodeTiled_v12000 fn, TMap *out, void *base, 
     return true;
 }
 
-template <typename T>
 static bool encode_state(PFN_cuTensorMapEncodeTiled_v12000 fn, const felbm_state *s, TMap maps[6]) {
+    using T = float;
     using PH = PairTile<T, kHD>;
     using PG = PairTile<T, 1>;
     const uint64_t nx = (uint64_t)s->mesh->sinfo.nx, ny = (uint64_t)s->mesh->sinfo.ny;
@@ -89,7 +89,7 @@ void lattice_tmaps(felbm_state *s) {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encoder();
     if (!fn) return;
     TMap maps[6];
-    if (!encode_state<float>(fn, s, maps)) return;
+    if (!encode_state(fn, s, maps)) return;
     TMap *d = nullptr;
     if (cudaMalloc((void **)&d, sizeof(maps)) != cudaSuccess) {
         cudaGetLastError();
