@@ -53,7 +53,8 @@ struct NvtxRange {
 };
 
 // ---- programmatic dependent launch -----------------------------------------
-// The kernels of a step are launched with programmatic stream serialisation:
+// The kernels of a step are launched with programmatic stream serialisation
+// (batches in FP64 and those that walk their tiles apart, plain launches):
 // a kernel may start while its predecessor drains, reads only what no kernel
 // writes (mesh tables) before pdl_wait(), and everything else after it.
 // pdl_wait() returns once the predecessor has completed, which itself waited
@@ -311,7 +312,9 @@ __device__ __forceinline__ int32_t ell_get(double w) { return __double2int_rn(w)
 // each(row, fn) calls fn(j, ax, ay, bxx, bxy, byy) for all of them, in
 // chunks.  Within a chunk the code has no branch, so that all its gathers are
 // in flight at once: a pass waits for one L2 access per chunk and not per
-// neighbour.
+// neighbour.  Chunks of 4 in FP32, 2 in FP64 (jittered Delaunay, us a step,
+// chunks of 4 / 2, twice and half as long: FP32 256 x 256 10.8, 12.8, 12.0, 600
+// x 600 62, 75, 64; FP64 153, 152, 161 and 770, 762, 802).
 template <typename T>
 struct DevELL {
     static constexpr int kChunk = sizeof(T) == 4 ? 4 : 2;

@@ -120,7 +120,9 @@ struct DevELL3 {
     }
     // Entries g, g + kSplitGroups, ... of the row of node i: the first kPart of them are
     // read by part_row (no kernel writes them), with the recovery
-    // coefficients only.
+    // coefficients only.  4 in FP32, 2 in FP64 (jittered tetrahedra 12^3, 28^3,
+    // 40^3, 56^3 FP32 16.1, 19.4, 38.4, 122 us a step, with 6 15.8, 19.0, 37.8,
+    // 121, with 2 17.0, 20.3, 36.8, 120; FP64 40^3 581, with 4 601, with 1 570).
     static constexpr int kPart = sizeof(T) == 4 ? 4 : 2, kGroups = kSplitGroups;
     struct PartRow {
         size_t p;
@@ -976,7 +978,7 @@ __global__ void __launch_bounds__(kSplitBlock, sizeof(T) == 4 ? 4 : 2)
     k_collide3_split(const __grid_constant__ Collide3Args<T, Topo> A) {
     // moments of g by group; grad mu in [4 ..][0]; the groups' h increments in [5 ..][1 ..]
     __shared__ T part[7][kSplitGroups][kSplitNodes];
-    // FP64: one group forms the scalars of a node for all four (its pipe
+    // FP64: one group forms the scalars of a node for all three (its pipe
     // bounds the pass; in FP32 each group forms them, a barrier less)
     constexpr bool kShare = sizeof(T) == 8;
     const int l = threadIdx.x % kSplitNodes, grp = threadIdx.x / kSplitNodes;

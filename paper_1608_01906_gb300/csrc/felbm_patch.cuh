@@ -16,8 +16,9 @@
 // order (k_grad, k_mu, k_collide), so both give the same results bit for bit.
 //
 // What bounds it: latency below about 10^5 nodes (one wave of blocks; three
-// dependent gathers and four barriers), the rows' and populations' bytes
-// above (about 370 of each node's, read and written).  Streaming h on rings
+// dependent gathers and four barriers), bytes above (about 450 of rows a node
+// in the two launches, 190 in k_rho, 260 here, beside 220 of populations, h*
+// and rho).  Streaming h on rings
 // <= 3 here too, in one launch, redid the costliest pass 1.9 times and waited
 // for its rows' coefficients in each stage: 24.5 us a step against 10.7 on a
 // 256 x 256 jittered Delaunay mesh (FP32), 270 against 159 on 1024 x 1024.
