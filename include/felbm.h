@@ -268,7 +268,8 @@ int felbm_batch_create(felbm_state *const *states, int32_t n_states, uint32_t fl
 int felbm_batch_step(felbm_batch *batch, int64_t n_steps);
 int felbm_batch_sync(felbm_batch *batch);
 /* Chosen configuration and counters; any output pointer may be NULL.
- * tile_order: 0 mesh-major, 1 interleaved across meshes. */
+ * tile_order: 0 mesh-major, 1 interleaved across meshes.  n_tiles: in FP64 the
+ * blocks of a pass (64 nodes each). */
 int felbm_batch_info(const felbm_batch *batch, int32_t *blocks_per_sm, int32_t *tile_order,
                      int32_t *n_tiles, int64_t *launches, double *tuned_ms_per_step);
 void felbm_batch_destroy(felbm_batch *batch);

@@ -94,8 +94,9 @@ def mesh_bytes(side):
 
 
 # Batch memory outside the states and meshes: per run a share of the tile
-# list (one 16-byte record per 32 x 8 tile), its descriptor and its 768
-# bytes of tensor maps; per batch the launch counters and the autotuner's
+# list (8-byte records, one per 32 x 8 tile in FP32, ragged ones included by
+# the factor of 2, one per 64 nodes in FP64), its descriptor and its 768 bytes
+# of tensor maps; per batch the launch counters and the autotuner's
 # buffers.
 BATCH_RUN_BYTES = 4096
 BATCH_FIXED_BYTES = 1 << 20
@@ -103,7 +104,8 @@ BATCH_FIXED_BYTES = 1 << 20
 
 def run_bytes(side, precision="fp32"):
     """Device bytes a run adds to a batch besides its mesh."""
-    return state_bytes(side, precision) + (side * side // 256 + 1) * 16 + BATCH_RUN_BYTES
+    tiles = (side * side // 256 + 1) * (16 if precision == "fp32" else 32)
+    return state_bytes(side, precision) + tiles + BATCH_RUN_BYTES
 
 
 def problem_for(req: Request):
