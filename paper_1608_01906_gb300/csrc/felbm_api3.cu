@@ -110,7 +110,7 @@ static DevLattice3<T> dev_lat3(const felbm_mesh *m, double dt) {
             for (int c = 0; c < 3; ++c) d.k.a[k][o][c] = (T)cf[c];
         }
     d.k.s12 = (T)(L.c[0][0][0] / kuhn_w(0, 0));
-    d.uni = kuhn_uniform(L) ? 1 : 0;
+    d.tables = !kuhn_uniform(L) ? 2 : d.walls;
     return d;
 }
 
@@ -250,7 +250,7 @@ static void step3(felbm_state *s, const Topo &d, const Fields3<T> &F, const Phys
     sl = prof_begin(s, 3);
     if constexpr (Topo::kLattice) {
         if (sizeof(T) == 4 || !split)
-            launch_pdl(d.uni ? k_collide3_node<T, true> : k_collide3_node<T, false>, nblocks3(m->n_nodes, 128), 128, 0,
+            launch_pdl(d.tables < 2 ? k_collide3_node<T, true> : k_collide3_node<T, false>, nblocks3(m->n_nodes, 128), 128, 0,
                        m->stream, A);
         else if constexpr (sizeof(T) == 8)
             launch_pdl(k_collide3_split<T, Topo>, nblocks3(m->n_nodes, kSplitNodes), kSplitBlock, 0, m->stream, A);

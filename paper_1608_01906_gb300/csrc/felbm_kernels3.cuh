@@ -187,7 +187,8 @@ struct DevLattice3 {
     static constexpr bool kLattice = true;
     int32_t n, nx, ny, nz;
     int32_t walls;
-    int32_t uni;  // the interior recovery weights are the integers kuhn_w times k.s12 (see kuhn_uniform)
+    int32_t tables;  // layers whose recovery weights are not the integers kuhn_w times k.s12: 0 none, 1 the wall
+                     // layers, 2 all (see kuhn_uniform)
     Lat3Coef<T> k;
 #ifdef __CUDACC__
     __device__ __forceinline__ int kind_of(int32_t i) const {
@@ -459,7 +460,7 @@ struct Col3 {
     int32_t pl[LZ + 2];  // first nodes of the planes z0 - 1 .. z0 + LZ (wrapped)
     int32_t z0, n;
     int count;           // nodes of the column in the lattice
-    bool table;          // its nodes take the tables: some are of a wall layer, or the lattice is not uniform
+    bool table;          // its nodes take the tables: some are of a layer of m.tables
     // false: no column of the lattice
     template <typename T>
     __device__ __forceinline__ bool set(const DevLattice3<T> &m) {
@@ -495,7 +496,7 @@ struct Col3 {
             z = z + 1 == m.nz ? 0 : z + 1;
         }
         count = m.nz - z0 < LZ ? m.nz - z0 : LZ;
-        table = !m.uni || (m.walls && (z0 == 0 || z0 + LZ >= m.nz));
+        table = m.tables && (m.tables == 2 || z0 == 0 || z0 + LZ >= m.nz);
         return true;
     }
     // node l of the column
@@ -1077,7 +1078,7 @@ __global__ void __launch_bounds__(kSplitBlock, sizeof(T) == 4 ? 4 : 2)
 
 // (all loads before the first store: interleaved with them the pass took
 // 232 us, not 172, on a 128^3 lattice in FP32)
-// UNI: the lattice's uni (read here instead it cost 1 % of a step).
+// UNI: the interior takes the integer weights (read here instead it cost 1 % of a step).
 template <typename T, bool UNI>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 1)
     k_collide3_node(const __grid_constant__ Collide3Args<T, DevLattice3<T>> A) {
